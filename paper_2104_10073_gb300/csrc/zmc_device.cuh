@@ -313,12 +313,21 @@ struct QuintUnroll {
 // Quints per accumulation block: a lane's shifted sums never span more than
 // 5 * kBlockQuints samples, which bounds their rounding error for any chunk length.
 constexpr uint32_t kBlockQuints = 13;
+
+// FAST: every sample of the chunk exists and one Philox prefix serves it (its block
+// indices share their high word).  Most rows end inside a chunk (a budget of 10^4
+// samples is less than one), so the other form matters too: it draws from the
+// prefix as well and checks bounds only in the step in which some lane runs out; a
+// chunk whose block index passes a multiple of 2^32 (crossing) forms every block's
+// whole counter.  Measured against whole counters and checks in every step: 5000
+// rows of 16384 samples 248 -> 222 us (abs-linear, 3-D), 506 -> 472 us (Gaussian,
+// 5-D); 12000 rows of 5000 samples 196 -> 176 us (abs-linear, 3-D).
 template <int FAM, int D, int G, bool FAST>
 __device__ __forceinline__ void run_chunk(const FnDev *__restrict__ fn, uint64_t chunk,
-                                          uint32_t Q, uint32_t lane) {
+                                          uint32_t Q, uint32_t lane, bool crossing) {
   Eval<FAM, D, G> ev;
   ev.load(fn);
-  const RoundKeys rk = make_round_keys(fn->key0, fn->key1);
+  const uint32_t key0 = fn->key0, key1 = fn->key1;
   const uint32_t sid = fn->stream_id;
   const uint64_t chunk_samples = chunk_samples_of(Q);
   const uint64_t s0 = chunk * chunk_samples;
@@ -327,7 +336,8 @@ __device__ __forceinline__ void run_chunk(const FnDev *__restrict__ fn, uint64_t
   const uint64_t quint0 = (fn->s_off + s0) / kQuint;  // s_off is a multiple of 5
   const uint64_t block0 = quint0 * D;
   const uint32_t base_lo0 = static_cast<uint32_t>(block0) + lane * D;
-  const StreamPrefix sp = make_stream_prefix(rk, sid, static_cast<uint32_t>(block0 >> 32));
+  const StreamPrefix sp = make_stream_prefix(make_round_keys(key0, key1), sid,
+                                             static_cast<uint32_t>(block0 >> 32));
 
   // running (n, mean, M2) of the lane, merged from blocks of kBlockQuints quints
   float n = 0.0f, mean = 0.0f, m2 = 0.0f;
@@ -345,10 +355,10 @@ __device__ __forceinline__ void run_chunk(const FnDev *__restrict__ fn, uint64_t
       const uint32_t ql = lane + 32u * j;
       if (!FAST && kQuint * ql >= nc) break;
       uint32_t r[5 * D];
-      if (FAST)
+      if (FAST || !crossing)
         gen_quint_fast<D>(base_lo0 + 32u * D * j, sp, r);
       else
-        gen_quint<D>(quint0 + ql, sid, rk, r);
+        gen_quint<D>(quint0 + ql, sid, make_round_keys(key0, key1), r);
       float f[5];
       eval_quint<D>(ev, r, f);
       if (j == jb) {
@@ -365,7 +375,8 @@ __device__ __forceinline__ void run_chunk(const FnDev *__restrict__ fn, uint64_t
         s2p = __ffma2_rn(d23, d23, s2p);
         const float d4 = f[4] - K;
         s2 = fmaf(d4, d4, s2);
-      } else if (FAST) {
+      } else if (FAST || 32u * kQuint * (j + 1) <= nc) {  // every lane's quint is whole
+        if (!FAST) cnt += kQuint;
         s1 += ((f[0] + f[1]) + (f[2] + f[3])) + f[4];
 #pragma unroll
         for (int t = 0; t < 5; ++t) {
@@ -411,9 +422,9 @@ __device__ __forceinline__ void run_item(const FnDev *__restrict__ fn, uint64_t 
   const uint64_t b_first = ((fn->s_off + s0) / kQuint) * D;
   const uint64_t b_last = b_first + (chunk_samples / kQuint) * D - 1;
   if (full && (b_first >> 32) == (b_last >> 32))
-    run_chunk<FAM, D, G, true>(fn, chunk, Q, lane);
+    run_chunk<FAM, D, G, true>(fn, chunk, Q, lane, false);
   else
-    run_chunk<FAM, D, G, false>(fn, chunk, Q, lane);
+    run_chunk<FAM, D, G, false>(fn, chunk, Q, lane, (b_first >> 32) != (b_last >> 32));
 }
 
 // Variant lists (family, dimension, polynomial degree or Gaussian form).
