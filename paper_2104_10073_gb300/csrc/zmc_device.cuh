@@ -310,9 +310,14 @@ struct QuintUnroll {
 #define ZMC_PASTE2(a, b) a##b
 #define ZMC_PASTE(a, b) ZMC_PASTE2(a, b)
 #define ZMC_FAMILY_OPS(name) ZMC_PASTE(name, ZMC_PASTE(U, ZMC_FAM_UNROLL))
-// Quints per accumulation block: a lane's shifted sums never span more than
-// 5 * kBlockQuints samples, which bounds their rounding error for any chunk length.
-constexpr uint32_t kBlockQuints = 13;
+
+// The part of a chunk that a warp takes: steps [j0, j1), all of them (part null: the
+// warp writes the chunk's record) or one accumulation block, whose 32 lane
+// summaries (mean, M2) go to part.
+struct Span {
+  uint32_t j0, j1;
+  float2 *part;
+};
 
 // FAST: every sample of the chunk exists and one Philox prefix serves it (its block
 // indices share their high word).  Most rows end inside a chunk (a budget of 10^4
@@ -324,7 +329,8 @@ constexpr uint32_t kBlockQuints = 13;
 // 5-D); 12000 rows of 5000 samples 196 -> 176 us (abs-linear, 3-D).
 template <int FAM, int D, int G, bool FAST>
 __device__ __forceinline__ void run_chunk(const FnDev *__restrict__ fn, uint64_t chunk,
-                                          uint32_t Q, uint32_t lane, bool crossing) {
+                                          uint32_t Q, uint32_t lane, const Span span,
+                                          bool crossing) {
   Eval<FAM, D, G> ev;
   ev.load(fn);
   const uint32_t key0 = fn->key0, key1 = fn->key1;
@@ -341,8 +347,8 @@ __device__ __forceinline__ void run_chunk(const FnDev *__restrict__ fn, uint64_t
 
   // running (n, mean, M2) of the lane, merged from blocks of kBlockQuints quints
   float n = 0.0f, mean = 0.0f, m2 = 0.0f;
-  for (uint32_t jb = 0; jb < Q; jb += kBlockQuints) {
-    const uint32_t je = jb + kBlockQuints < Q ? jb + kBlockQuints : Q;
+  for (uint32_t jb = span.j0; jb < span.j1; jb += kBlockQuints) {
+    const uint32_t je = jb + kBlockQuints < span.j1 ? jb + kBlockQuints : span.j1;
     float K = 0.0f, s1 = 0.0f, s2 = 0.0f;
     // families that ask for it (Eval::kPackedSums) sum full quints in packed
     // pairs: samples (0, 1) and (2, 3) as pairs, 4 alone (the others keep the
@@ -405,26 +411,30 @@ __device__ __forceinline__ void run_chunk(const FnDev *__restrict__ fn, uint64_t
       const float mb = __fdiv_rn(s1, nb);
       const float dk = __fsub_rn(mb, K);
       const float m2b = fmaxf(fmaf(__fmul_rn(-nb, dk), dk, s2), 0.0f);
-      chan_step(n, mean, m2, nb, mb, m2b);
+      if (span.part)
+        span.part[lane] = make_float2(mb, m2b);
+      else
+        chan_step(n, mean, m2, nb, mb, m2b);
     }
     if (!FAST && cnt < kQuint * (je - jb)) break;
   }
+  if (span.part) return;
   warp_chan_merge(n, mean, m2);
   if (lane == 0) fn->rec[chunk] = make_float2(mean, m2);
 }
 
 template <int FAM, int D, int G>
 __device__ __forceinline__ void run_item(const FnDev *__restrict__ fn, uint64_t chunk,
-                                         uint32_t Q, uint32_t lane) {
+                                         uint32_t Q, uint32_t lane, const Span span) {
   const uint64_t chunk_samples = chunk_samples_of(Q);
   const uint64_t s0 = chunk * chunk_samples;
   const bool full = fn->n_samples - s0 >= chunk_samples;
   const uint64_t b_first = ((fn->s_off + s0) / kQuint) * D;
   const uint64_t b_last = b_first + (chunk_samples / kQuint) * D - 1;
   if (full && (b_first >> 32) == (b_last >> 32))
-    run_chunk<FAM, D, G, true>(fn, chunk, Q, lane, false);
+    run_chunk<FAM, D, G, true>(fn, chunk, Q, lane, span, false);
   else
-    run_chunk<FAM, D, G, false>(fn, chunk, Q, lane, (b_first >> 32) != (b_last >> 32));
+    run_chunk<FAM, D, G, false>(fn, chunk, Q, lane, span, (b_first >> 32) != (b_last >> 32));
 }
 
 // Variant lists (family, dimension, polynomial degree or Gaussian form).
@@ -442,31 +452,40 @@ __device__ __forceinline__ void run_item(const FnDev *__restrict__ fn, uint64_t 
 #define ZMC_GAUSS_VARIANTS(X) ZMC_VARIANTS_DIM(X, ZMC_GAUSS, 0) ZMC_VARIANTS_DIM(X, ZMC_GAUSS, 1)
 // switch cases of dispatch_item / dispatch_eval
 #define ZMC_ITEM_CASE(F, D, G) \
-  case variant_code(F, D, G): run_item<F, D, G>(fn, chunk, Q, lane); break;
+  case variant_code(F, D, G): run_item<F, D, G>(fn, chunk, Q, lane, span); break;
 #define ZMC_EVAL_CASE(F, D, G) \
   case variant_code(F, D, G): eval_range<F, D, G>(fn, s_begin, count, out); break;
 
+// The entry that holds `item`, by the whole warp: each step probes 32 evenly spaced
+// entries at once, so 10^3 entries take two dependent loads and 10^4 three (a
+// binary search takes 10 and 14, each an L2 access of its own, and on a launch of
+// one chunk or block per row every item pays it).  Invariant: entries[lo] begins at
+// or before the item, entries[hi] (if any) after it.
 __device__ __forceinline__ uint32_t find_entry(const Entry *__restrict__ entries, uint32_t ne,
-                                               uint64_t item, uint32_t hint) {
-  if (hint < ne && entries[hint].item_begin <= item &&
-      (hint + 1 == ne || entries[hint + 1].item_begin > item))
-    return hint;
-  uint32_t lo = 0, hi = ne;  // invariant: entries[lo].item_begin <= item < entries[hi]
-  if (hint < ne && entries[hint].item_begin <= item) lo = hint;
+                                               uint64_t item, uint32_t lane) {
+  uint32_t lo = 0, hi = ne;
   while (hi - lo > 1) {
-    const uint32_t mid = (lo + hi) >> 1;
-    if (entries[mid].item_begin <= item)
-      lo = mid;
-    else
-      hi = mid;
+    const uint32_t step = (hi - lo + 31u) / 32u;
+    const uint32_t at = lo + step * lane;
+    const uint32_t n = __popc(__ballot_sync(kFullMask, at < hi && entries[at].item_begin <= item));
+    lo += step * (n - 1u);  // lane 0 probes lo itself: n >= 1
+    if (lo + step < hi) hi = lo + step;
   }
   return lo;
+}
+
+// Samples of a chunk of an integrand.
+__device__ __forceinline__ uint32_t samples_of(const FnDev *__restrict__ fn, uint64_t chunk,
+                                               uint32_t Q) {
+  const uint64_t left = fn->n_samples - chunk * chunk_samples_of(Q);
+  return static_cast<uint32_t>(left < chunk_samples_of(Q) ? left : chunk_samples_of(Q));
 }
 
 // One work item (chunk) of an integrand of family FAM: switch on its variant to
 // the specialised run_item.  Specialised per family.
 template <int FAM>
-__device__ void dispatch_item(const FnDev *fn, uint64_t chunk, uint32_t Q, uint32_t lane);
+__device__ void dispatch_item(const FnDev *fn, uint64_t chunk, uint32_t Q, uint32_t lane,
+                              const Span span);
 
 // Persistent, one kernel per family (so each gets the register budget of its own
 // variants): each warp takes the next work item of its family from a global
@@ -525,25 +544,48 @@ struct HdrSlot {
   static constexpr int value = FAM < 4 ? FAM : 0;
 };
 
+// A launch hands out whole chunks and, at its end, the last hdr->split of them by
+// accumulation blocks (13 quints a lane, eight to a chunk at Q = 104): as long as
+// chunks last every warp is busy, but a launch of few chunks, and the end of a
+// launch whose chunks differ in length, would leave most of the chip idle for up to
+// a chunk's time (60 .. 190 us at Q = 104).  A block's lane summaries go to the
+// launch's scratch, and zmc_combine_kernel makes the chunks' records of them.
+// (Counting a chunk's blocks and combining them here, in the warp that completes the
+// count, kept so much state alive over the chunk's body that whole chunks of the
+// polynomial kernel slowed down by 3%; drawing the next item before the body, to
+// hide the counter's latency, took items from idle warps: 100 rows of 10^5 samples
+// 116 instead of 65 us.)
 template <int FAM>
 __device__ __forceinline__ void batched_loop(const Entry *__restrict__ entries,
                                              LaunchHdr *__restrict__ hdr) {
   constexpr int kSlot = HdrSlot<FAM>::value;
   const uint32_t lane = threadIdx.x & 31u;
   const unsigned long long begin = hdr->item_begin[kSlot];
-  const unsigned long long count = hdr->item_end[kSlot] - begin;
   const uint32_t ne = hdr->n_entries;
   const uint32_t Q = hdr->quints_per_lane;
-  uint32_t e = 0;
+  const uint32_t split = hdr->split[kSlot];
+  const unsigned long long whole = hdr->item_end[kSlot] - begin - split;
   for (;;) {
     unsigned long long k = 0;
     if (lane == 0) k = atomicAdd(&hdr->counter[kSlot], 1ull);
     k = __shfl_sync(kFullMask, k, 0);
-    if (k >= count) break;
+    Span span = {0u, Q, nullptr};
+    if (k >= whole) {
+      const uint32_t nb = chunk_blocks(Q);
+      const unsigned long long u = k - whole;
+      if (u >= static_cast<unsigned long long>(split) * nb) break;
+      const uint32_t t = static_cast<uint32_t>(u) / nb;
+      k = whole + t;
+      span.j0 = (static_cast<uint32_t>(u) - t * nb) * kBlockQuints;
+      span.j1 = span.j0 + kBlockQuints < Q ? span.j0 + kBlockQuints : Q;
+      span.part = hdr->part[kSlot] + static_cast<size_t>(u) * 32u;
+    }
     const uint64_t item = begin + k;
-    e = find_entry(entries, ne, item, e);
-    const Entry en = entries[e];
-    dispatch_item<FAM>(en.fn, en.chunk_begin + (item - en.item_begin), Q, lane);
+    const Entry en = entries[find_entry(entries, ne, item, lane)];
+    const uint64_t chunk = en.chunk_begin + (item - en.item_begin);
+    // a block after the chunk's last sample holds nothing
+    if (span.j0 && samples_of(en.fn, chunk, Q) <= chunk_samples_of(span.j0)) continue;
+    dispatch_item<FAM>(en.fn, chunk, Q, lane, span);
   }
 }
 

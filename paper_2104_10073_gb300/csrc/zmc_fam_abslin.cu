@@ -61,7 +61,7 @@ struct Eval<ZMC_ABSLIN, D, G> {
 
 template <>
 __device__ void dispatch_item<ZMC_ABSLIN>(const FnDev *fn, uint64_t chunk, uint32_t Q,
-                                      uint32_t lane) {
+                                      uint32_t lane, const Span span) {
   switch (fn->variant) {
     ZMC_ABSLIN_VARIANTS(ZMC_ITEM_CASE)
     ZMC_VARIANTS_DIM(ZMC_ITEM_CASE, ZMC_ABSLIN, 1)

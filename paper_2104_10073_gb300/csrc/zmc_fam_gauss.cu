@@ -123,7 +123,7 @@ struct Eval<ZMC_GAUSS, D, G> {
 
 template <>
 __device__ void dispatch_item<ZMC_GAUSS>(const FnDev *fn, uint64_t chunk, uint32_t Q,
-                                      uint32_t lane) {
+                                      uint32_t lane, const Span span) {
   switch (fn->variant) {
     ZMC_GAUSS_VARIANTS(ZMC_ITEM_CASE)
     default:

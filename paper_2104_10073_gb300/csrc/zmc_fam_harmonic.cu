@@ -171,7 +171,7 @@ struct Eval<ZMC_HARMONIC, D, G> {
 
 template <>
 __device__ void dispatch_item<ZMC_HARMONIC>(const FnDev *fn, uint64_t chunk, uint32_t Q,
-                                      uint32_t lane) {
+                                      uint32_t lane, const Span span) {
   switch (fn->variant) {
     ZMC_HARMONIC_VARIANTS(ZMC_ITEM_CASE)
     ZMC_HARMONIC_EQUAL_VARIANTS(ZMC_ITEM_CASE)

@@ -108,7 +108,7 @@ struct Eval<ZMC_POLY, D, G>
 
 template <>
 __device__ void dispatch_item<ZMC_POLY>(const FnDev *fn, uint64_t chunk, uint32_t Q,
-                                      uint32_t lane) {
+                                      uint32_t lane, const Span span) {
   switch (fn->variant) {
     ZMC_POLY_VARIANTS(ZMC_ITEM_CASE)
     ZMC_POLY_ROOT_VARIANTS(ZMC_ITEM_CASE)

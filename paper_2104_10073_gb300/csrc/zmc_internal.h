@@ -99,6 +99,13 @@ struct alignas(16) FnDev {
 };
 static_assert(sizeof(FnDev) == 384, "FnDev layout");
 
+// Quints per accumulation block: a lane's shifted sums never span more than
+// 5 * kBlockQuints samples, which bounds their rounding error for any chunk length.
+constexpr uint32_t kBlockQuints = 13;
+__host__ __device__ constexpr uint32_t chunk_blocks(uint32_t quints_per_lane) {
+  return (quints_per_lane + kBlockQuints - 1) / kBlockQuints;
+}
+
 // A contiguous run of chunks of one integrand inside one persistent launch.
 struct Entry {
   uint64_t item_begin;   // first work-item index of this run in the launch
@@ -119,6 +126,11 @@ struct LaunchHdr {
   uint32_t n_merge;                  // integrands to merge after this launch
   uint32_t quints_per_lane;          // chunk = 160 * quints_per_lane samples
   uint32_t pad;
+  // The last split[f] items of family f are handed out by accumulation blocks;
+  // block b of item t of them has its 32 lane summaries at
+  // part[f][32 (blocks per chunk t + b)].
+  uint32_t split[4];
+  float2 *part[4];
 };
 
 // FP64 descriptor of the plain per-integrand kernel (passed by value).
@@ -159,6 +171,9 @@ constexpr int kMaxUnroll = 2;
 // cudaError_t; an unknown family or unroll gives cudaErrorInvalidValue.
 cudaError_t launch_batched(int family, const Entry *entries, LaunchHdr *hdr, unsigned grid,
                            unsigned block, cudaStream_t stream, int unroll = 1);
+// The records of a launch's split chunks (`chunks` of them over the families).
+cudaError_t launch_combine(const Entry *entries, const LaunchHdr *hdr, uint64_t chunks, int sms,
+                           cudaStream_t stream);
 cudaError_t launch_merge(const FnDev *const *fns, const LaunchHdr *hdr, unsigned grid,
                          cudaStream_t stream);
 cudaError_t launch_plain(const PlainFn &fn, double *block_rec, unsigned grid,

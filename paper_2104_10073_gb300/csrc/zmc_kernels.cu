@@ -22,10 +22,72 @@
 // No tensor cores and no TMA: the path is integer and FP32 arithmetic on the FMA,
 // ALU and MUFU pipes, with a few KB of descriptor reads and 8 bytes written per
 // 160 * quints_per_lane samples.
+#include <algorithm>
+#include <atomic>
+
 #include "zmc_device.cuh"
 
 namespace zmc {
 namespace {
+
+// ---------------------------------------------------------------- split chunks
+// Samples of a lane's steps [jb, je) in a chunk of nc samples.
+__device__ __forceinline__ uint32_t lane_block_samples(uint32_t nc, uint32_t lane, uint32_t jb,
+                                                       uint32_t je) {
+  const uint32_t nq = nc / kQuint, rest = nc - kQuint * nq;  // whole quints, samples after them
+  const uint32_t jl = nq > lane ? (nq - lane + 31u) / 32u : 0u;  // the lane's whole quints
+  const uint32_t whole = jl <= jb ? 0u : (jl < je ? jl : je) - jb;
+  const uint32_t j = nq / 32u;
+  return kQuint * whole + (lane == nq % 32u && j >= jb && j < je ? rest : 0u);
+}
+
+// The record of a chunk from its blocks' lane summaries: the same steps, in the
+// same order, as a warp that took the whole chunk.  Eight blocks (a chunk at the
+// default Q = 104) are loaded at a time, so that their latencies overlap.
+__device__ __forceinline__ void combine_blocks(const FnDev *__restrict__ fn, uint64_t chunk,
+                                               uint32_t nc, uint32_t Q, uint32_t lane,
+                                               const float2 *part) {
+  float n = 0.0f, mean = 0.0f, m2 = 0.0f;
+  for (uint32_t j0 = 0; j0 < Q && chunk_samples_of(j0) < nc; j0 += 8 * kBlockQuints) {
+    uint32_t cnt[8];
+    float2 b[8];
+#pragma unroll
+    for (uint32_t i = 0; i < 8; ++i) {
+      const uint32_t jb = j0 + i * kBlockQuints;
+      const uint32_t je = jb + kBlockQuints < Q ? jb + kBlockQuints : Q;
+      cnt[i] = jb < Q ? lane_block_samples(nc, lane, jb, je) : 0u;
+      if (cnt[i]) b[i] = __ldcg(part + 32u * (jb / kBlockQuints) + lane);
+    }
+#pragma unroll
+    for (uint32_t i = 0; i < 8; ++i)
+      if (cnt[i]) chan_step(n, mean, m2, static_cast<float>(cnt[i]), b[i].x, b[i].y);
+  }
+  __syncwarp();
+  warp_chan_merge(n, mean, m2);
+  if (lane == 0) fn->rec[chunk] = make_float2(mean, m2);
+}
+
+// One warp per split chunk of a launch (LaunchHdr::split), of any family: a few
+// loads and ~13 dependent merge steps each, so it is bound by latency; 304 blocks
+// hold all of a launch's warps at once.
+__global__ void __launch_bounds__(256) zmc_combine_kernel(const Entry *__restrict__ entries,
+                                                          const LaunchHdr *__restrict__ hdr) {
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
+  const uint32_t Q = hdr->quints_per_lane;
+  uint32_t w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  for (int f = 0; f < 4; ++f) {
+    const uint32_t split = hdr->split[f];
+    for (; w < split; w += nwarps) {
+      const uint64_t item = hdr->item_end[f] - split + w;
+      const Entry en = entries[find_entry(entries, hdr->n_entries, item, lane)];
+      const uint64_t chunk = en.chunk_begin + (item - en.item_begin);
+      combine_blocks(en.fn, chunk, samples_of(en.fn, chunk, Q), Q, lane,
+                     hdr->part[f] + static_cast<size_t>(w) * 32u * chunk_blocks(Q));
+    }
+    w -= split;  // the next family's chunks go on with the next warp
+  }
+}
 
 // ---------------------------------------------------------------- FP64 merge
 // One warp per integrand.  With chunk summaries (n_c, m_c, M2_c):
@@ -153,9 +215,27 @@ cudaError_t launch_merge(const FnDev *const *fns, const LaunchHdr *hdr, unsigned
   return cudaGetLastError();
 }
 
+cudaError_t launch_combine(const Entry *entries, const LaunchHdr *hdr, uint64_t chunks, int sms,
+                           cudaStream_t stream) {
+  if (chunks == 0) return cudaSuccess;
+  const uint64_t blocks = std::min<uint64_t>((chunks + 7) / 8, 2ull * static_cast<unsigned>(sms));
+  zmc_combine_kernel<<<static_cast<unsigned>(blocks), 256, 0, stream>>>(entries, hdr);
+  return cudaGetLastError();
+}
+
+// Kept per kernel and block size: every device this library runs on is the same
+// part, and the query is on the path of each blocking call.
 int batched_max_blocks_per_sm(int family, int block, int unroll) {
   const FamilyOps *ops = ops_of(family, unroll);
-  return ops ? ops->max_blocks_per_sm(block) : 0;
+  if (!ops || block < 32 || block > 1024) return 0;
+  static std::atomic<int> known[kMaxUnroll][4][33];
+  std::atomic<int> &k = known[unroll - 1][family][block / 32];
+  int n = k.load(std::memory_order_relaxed);
+  if (n == 0) {
+    n = ops->max_blocks_per_sm(block);
+    k.store(n, std::memory_order_relaxed);
+  }
+  return n;
 }
 
 int batched_regs_per_thread(int family, int unroll) {

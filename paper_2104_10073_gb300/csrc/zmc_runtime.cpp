@@ -463,6 +463,42 @@ unsigned family_grid(const zmc_ctx *ctx, int family, uint64_t items, int unroll)
   return grid_for(ctx, family, ctx->shape.block, ctx->shape.blocks_per_sm[family], items, unroll);
 }
 
+// How many of a launch's last chunks are handed out by accumulation blocks
+// (LaunchHdr::split), given the warps it keeps resident.
+// A launch of fewer chunks than that spreads over the chip from its first block on:
+// 20 abs-linear chunks in 3-D 22.9 against 38.8 us whole (plan run, merge and launch
+// gaps included), 20 polynomials in 7-D 36 against 129 us, 1400 abs-linear chunks 75
+// against 92 us.  A block costs its draw, lookup and descriptor loads again, ~2.5 us
+// of latency, so chunks that are alike and nearly fill a whole number of warps per
+// scheduler stay whole (1216 chunks, two warps: 54 against 62 us; 2432, four: 93
+// against 110), and so do alike chunks in more than one wave, which end together
+// anyway (4864: 171 either way, 188 split).
+// Chunks that differ in cost (families, dimensions, polynomial degrees) leave a tail
+// of up to the longest chunk's time at the end and a CTA's slowest warp's time at
+// each change of family: one chunk per resident warp fills it (300 mixed rows 1117
+// against 1295 us, 64 mixed rows 295 against 386).
+// The lane summaries take 256 bytes a block, at most kSplitBytes a family (5 MB at
+// the default Q = 104).  None for chunks of one block.
+uint32_t split_chunks(uint64_t items, bool alike, uint64_t resident_warps, uint32_t quints) {
+  const uint64_t nb = chunk_blocks(quints), w = resident_warps;
+  if (nb < 2) return 0;
+  const bool fills = 5 * items > 4 * w || (5 * items > 2 * w && 2 * items <= w);
+  if (alike && fills) return 0;
+  return static_cast<uint32_t>(std::min({items, w, kSplitBytes / (nb * kPartBytes)}));
+}
+
+// Whole chunks and blocks of split ones.
+uint64_t launch_units(uint64_t items, uint32_t split, uint32_t quints) {
+  return items - split + static_cast<uint64_t>(split) * chunk_blocks(quints);
+}
+
+// Threads per block: `block`, less when the units do not fill one such block per
+// SM, so that few units take one SM each instead of sharing a few.
+unsigned spread_block(unsigned block, uint64_t units, int sms) {
+  while (block > 32 && (block / 64) * static_cast<uint64_t>(sms) >= units) block /= 2;
+  return block;
+}
+
 cudaError_t FamilyFork::init() {
   cudaError_t e = cudaEventCreateWithFlags(&fork, cudaEventDisableTiming);
   for (int k = 0; k < 3 && e == cudaSuccess; ++k) {
@@ -529,6 +565,8 @@ struct zmc_plan {
   LaunchHdr h_hdr{};
   uint64_t n_chunks = 0, n_samples = 0;
   uint64_t fam_items[4] = {0, 0, 0, 0};
+  uint64_t fam_units[4] = {0, 0, 0, 0};  // whole chunks and blocks of split ones
+  void *d_part = nullptr;  // lane summaries of the split chunks
   bool ranged = false;  // built by zmc_integrate_moments (no plain form)
   uint32_t quints = 0;  // chunk = 160 * quints samples
   unsigned unroll[4] = {1, 1, 1, 1};  // quint-loop unroll of each family kernel
@@ -541,15 +579,51 @@ struct zmc_plan {
   std::vector<void *> blocks;
 
   void *alloc(size_t bytes) {
-    void *p = ctx->arena.alloc(bytes);
+    void *p = arena_take(ctx, bytes);
     if (p) blocks.push_back(p);
     return p;
   }
   void release_all() {
     for (void *p : blocks) ctx->arena.release(p);
     blocks.clear();
+    if (d_part) {
+      ctx->arena.release(d_part);
+      ctx->split_plans.erase(this);
+      d_part = nullptr;
+    }
   }
 };
+
+namespace zmc {
+
+// Gives the scratch of every plan back to the arena: from the next run on, those
+// plans hand out whole chunks only.
+static void drop_splits(zmc_ctx *ctx) {
+  bool ok = true;
+  for (zmc_plan *p : ctx->split_plans) {
+    std::memset(p->h_hdr.split, 0, sizeof p->h_hdr.split);
+    ok = ok && cudaMemcpyAsync(p->d_hdr, &p->h_hdr, sizeof p->h_hdr, cudaMemcpyHostToDevice,
+                               ctx->stream) == cudaSuccess;
+  }
+  // launches already enqueued use the scratch
+  if (cudaStreamSynchronize(ctx->stream) != cudaSuccess || !ok) return;
+  for (zmc_plan *p : ctx->split_plans) {
+    ctx->arena.release(p->d_part);
+    p->d_part = nullptr;
+  }
+  ctx->split_plans.clear();
+}
+
+void *arena_take(zmc_ctx *ctx, size_t bytes) {
+  void *p = ctx->arena.alloc(bytes);
+  if (!p && !ctx->split_plans.empty()) {
+    drop_splits(ctx);
+    p = ctx->arena.alloc(bytes);
+  }
+  return p;
+}
+
+}  // namespace zmc
 
 namespace {
 
@@ -578,7 +652,7 @@ zmc_status plan_autotune(zmc_plan *plan) {
     if (hit != ctx->tune_cache.end()) {
       plan->block[f] = hit->second.block;
       plan->grid[f] = grid_for(ctx, f, hit->second.block, hit->second.blocks_per_sm,
-                               plan->fam_items[f], U);
+                               plan->fam_units[f], U);
       plan->tune_source[f] = 2;
       continue;
     }
@@ -594,7 +668,10 @@ zmc_status plan_autotune(zmc_plan *plan) {
     LaunchHdr th = plan->h_hdr;
     const uint64_t slice = std::min<uint64_t>(plan->fam_items[f],
                                               static_cast<uint64_t>(ctx->sms) * 64 * 32);
-    for (int g = 0; g < 4; ++g) th.item_end[g] = th.item_begin[g];
+    for (int g = 0; g < 4; ++g) {
+      th.item_end[g] = th.item_begin[g];
+      th.split[g] = 0;
+    }
     th.item_end[f] = th.item_begin[f] + slice;
     TuneChoice best;
     best.ms = 1e30f;
@@ -627,7 +704,7 @@ zmc_status plan_autotune(zmc_plan *plan) {
     }
     if (st != ZMC_OK) break;
     plan->block[f] = best.block;
-    plan->grid[f] = grid_for(ctx, f, best.block, best.blocks_per_sm, plan->fam_items[f], U);
+    plan->grid[f] = grid_for(ctx, f, best.block, best.blocks_per_sm, plan->fam_units[f], U);
     plan->tune_source[f] = 1;
     tune_cache_store(ctx, key, best);
   }
@@ -651,7 +728,7 @@ struct PlanChoice {
 
 zmc_status plan_build(zmc_ctx *ctx, const zmc_desc *desc, size_t n, zmc_plan **out,
                       const uint64_t *s_begin = nullptr, const uint64_t *s_end = nullptr,
-                      const PlanChoice *force = nullptr, bool wait_upload = true);
+                      const PlanChoice *force = nullptr, bool keep = true);
 void plan_free(zmc_plan *plan);
 zmc_status plan_enqueue(zmc_plan *plan, uint32_t stages);
 
@@ -687,7 +764,7 @@ zmc_status time_family(zmc_plan *plan, int f, int unroll, cudaEvent_t e0, cudaEv
   zmc_ctx *ctx = plan->ctx;
   cudaStream_t str = ctx->stream;
   const unsigned grid = grid_for(ctx, f, ctx->shape.block, ctx->shape.blocks_per_sm[f],
-                                 plan->fam_items[f], unroll);
+                                 plan->fam_units[f], unroll);
   float best = 1e30f;
   for (int rep = 0; rep < 3; ++rep) {
     cudaError_t e = cudaMemsetAsync(plan->d_hdr, 0, sizeof(plan->d_hdr->counter), str);
@@ -856,12 +933,12 @@ zmc_status choose_chunk(zmc_ctx *ctx, const zmc_desc *desc, size_t n, PlanChoice
 
 // ranges: optional [s_begin[i], s_end[i]) sample ranges (moments output).
 // force: a fixed chunk length and unroll, no autotuning (trial plans).
-// wait_upload = false: the caller's next use of the staging buffer is
-// stream-ordered after the upload (a device-to-host copy of results), so the
-// host need not wait for the upload here.
+// keep = false: the plan goes before the call returns, and the caller's next use of
+// the staging buffer is stream-ordered after the upload (a device-to-host copy of
+// results), so the host need not wait for the upload here.
 zmc_status plan_build(zmc_ctx *ctx, const zmc_desc *desc, size_t n, zmc_plan **out,
                       const uint64_t *s_begin, const uint64_t *s_end, const PlanChoice *force,
-                      bool wait_upload) {
+                      bool keep) {
   if (!desc || !out || n == 0) return set_error(ZMC_EINVAL, "need n >= 1 descriptors");
   if (n >= (1u << 31)) return set_error(ZMC_EINVAL, "too many descriptors");
   auto plan = std::make_unique<zmc_plan>();
@@ -929,6 +1006,24 @@ zmc_status plan_build(zmc_ctx *ctx, const zmc_desc *desc, size_t n, zmc_plan **o
   plan->d_out = static_cast<zmc_result *>(plan->alloc(n * sizeof(zmc_result)));
   plan->d_entries = static_cast<Entry *>(plan->alloc(ent_bytes));
   plan->d_merge = static_cast<const FnDev **>(plan->alloc(mrg_bytes));
+  // chunks of each family and how many of them are split
+  uint64_t fam_chunks[4] = {0, 0, 0, 0};
+  for (size_t i = 0; i < n; ++i) fam_chunks[desc[i].family] += nchunk[i];
+  uint32_t dmin = kMaxDim, dmax = 1, split[4], n_split = 0;
+  bool alike = true;  // one family, one degree, dimensions within a factor 3/2
+  for (size_t i = 0; i < n; ++i) {
+    dmin = std::min(dmin, desc[i].dim);
+    dmax = std::max(dmax, desc[i].dim);
+    alike = alike && desc[i].family == desc[0].family &&
+            (desc[i].family != ZMC_POLY || desc[i].deg == desc[0].deg);
+  }
+  alike = alike && 2 * dmax <= 3 * dmin;
+  for (int f = 0; f < 4; ++f) {
+    const int bps = batched_max_blocks_per_sm(f, 256, static_cast<int>(plan->unroll[f]));
+    split[f] = split_chunks(fam_chunks[f], alike,
+                            static_cast<uint64_t>(ctx->sms) * 8 * std::max(bps, 1), plan->quints);
+    n_split += split[f];
+  }
   plan->d_hdr = static_cast<LaunchHdr *>(plan->alloc(sizeof(LaunchHdr)));
   if (!plan->d_fns || !plan->d_rec || !plan->d_out || !plan->d_entries || !plan->d_merge ||
       !plan->d_hdr) {
@@ -977,10 +1072,29 @@ zmc_status plan_build(zmc_ctx *ctx, const zmc_desc *desc, size_t n, zmc_plan **o
   h.n_entries = static_cast<uint32_t>(n);
   h.n_merge = static_cast<uint32_t>(n);
   h.quints_per_lane = plan->quints;
+  // the scratch of the split chunks, the last thing taken from the arena: without
+  // room for it every chunk stays whole (arena_take takes it back when a later
+  // table needs the room; the serving scheduler cannot, so a plan of a serving
+  // context that outlives the call has none)
+  const size_t nb = chunk_blocks(plan->quints);
+  if (n_split && !(ctx->serving && keep))
+    plan->d_part = ctx->arena.alloc(n_split * nb * kPartBytes);
+  if (plan->d_part) {
+    ctx->split_plans.insert(plan.get());
+    auto *part = static_cast<float2 *>(plan->d_part);
+    for (int f = 0; f < 4; ++f) {
+      h.split[f] = split[f];
+      h.part[f] = part;
+      part += split[f] * nb * 32;
+    }
+  }
   for (int f = 0; f < 4; ++f) {
+    const int unroll = static_cast<int>(plan->unroll[f]);
     plan->fam_items[f] = h.item_end[f] - h.item_begin[f];
-    plan->block[f] = ctx->shape.block;
-    plan->grid[f] = family_grid(ctx, f, plan->fam_items[f], static_cast<int>(plan->unroll[f]));
+    plan->fam_units[f] = launch_units(plan->fam_items[f], h.split[f], plan->quints);
+    plan->block[f] = spread_block(ctx->shape.block, plan->fam_units[f], ctx->sms);
+    plan->grid[f] = grid_for(ctx, f, plan->block[f], ctx->shape.blocks_per_sm[f],
+                             plan->fam_units[f], unroll);
   }
   {
     double dim_samples[4][kMaxDim + 1] = {{0}};
@@ -1019,7 +1133,7 @@ zmc_status plan_build(zmc_ctx *ctx, const zmc_desc *desc, size_t n, zmc_plan **o
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(plan->d_hdr, s + fn_bytes + ent_bytes + mrg_bytes, sizeof h,
                         cudaMemcpyHostToDevice, str);
-  if (e == cudaSuccess && wait_upload) e = cudaStreamSynchronize(str);
+  if (e == cudaSuccess && keep) e = cudaStreamSynchronize(str);
   if (e != cudaSuccess) {
     plan->release_all();
     return ctx_cuda_fail(ctx, e, "plan upload");
@@ -1044,6 +1158,9 @@ zmc_status plan_enqueue(zmc_plan *plan, uint32_t stages) {
     for (int f = 0; f < 4; ++f) present[f] = plan->fam_items[f] > 0;
     ZMC_CUDA(ctx, launch_families(ctx->fork, plan->d_entries, plan->d_hdr, plan->grid,
                                   plan->block, present, str, plan->unroll));
+    uint64_t split = 0;
+    for (uint32_t s : plan->h_hdr.split) split += s;
+    ZMC_CUDA(ctx, launch_combine(plan->d_entries, plan->d_hdr, split, ctx->sms, str));
   }
   if (stages & ZMC_STAGE_MERGE) {
     const unsigned grid = static_cast<unsigned>(
@@ -1441,7 +1558,7 @@ zmc_status zmc_philox4x32_10(zmc_ctx *ctx, const uint32_t *ctr, const uint32_t *
   if (!ctr || !key || !out) return set_error(ZMC_EINVAL, "null argument");
   std::lock_guard<std::recursive_mutex> g(ctx->api_mu);
   const size_t bytes = n * 40;  // 16 ctr + 8 key + 16 out
-  char *d = static_cast<char *>(ctx->arena.alloc(bytes));
+  char *d = static_cast<char *>(arena_take(ctx, bytes));
   if (!d) return set_error(ZMC_ENOMEM, "arena full");
   st = ensure_stage(ctx, bytes);
   if (st == ZMC_OK) {
@@ -1477,7 +1594,7 @@ zmc_status zmc_philox_rate(zmc_ctx *ctx, uint64_t n_blocks, double *blocks_per_s
   const uint64_t per = std::max<uint64_t>(4, (n_blocks + threads * 4 - 1) / (threads * 4) * 4);
   if (per > 0xFFFFFFF0ull) return set_error(ZMC_EINVAL, "n_blocks too large for one wave");
   const uint32_t per_thread = static_cast<uint32_t>(per);
-  uint32_t *d = static_cast<uint32_t *>(ctx->arena.alloc(threads * sizeof(uint32_t)));
+  uint32_t *d = static_cast<uint32_t *>(arena_take(ctx, threads * sizeof(uint32_t)));
   if (!d) return set_error(ZMC_ENOMEM, "arena full");
   cudaEvent_t ev[2] = {nullptr, nullptr};
   cudaError_t e = cudaEventCreate(&ev[0]);
@@ -1512,7 +1629,7 @@ zmc_status zmc_eval_samples(zmc_ctx *ctx, const zmc_desc *desc, uint64_t s_begin
   if (st != ZMC_OK) return st;
   std::lock_guard<std::recursive_mutex> g(ctx->api_mu);
   const size_t bytes = sizeof(FnDev) + static_cast<size_t>(count) * 4;
-  char *d = static_cast<char *>(ctx->arena.alloc(bytes));
+  char *d = static_cast<char *>(arena_take(ctx, bytes));
   if (!d) return set_error(ZMC_ENOMEM, "arena full");
   st = ensure_stage(ctx, bytes);
   if (st == ZMC_OK) {

@@ -9,6 +9,7 @@
 #include <map>
 #include <memory>
 #include <mutex>
+#include <set>
 #include <string>
 #include <thread>
 #include <unordered_map>
@@ -114,6 +115,7 @@ struct zmc_ctx {
   std::map<std::string, zmc::TuneChoice> tune_cache;  // autotuner results by key
   std::atomic<bool> poisoned{false};
   std::recursive_mutex api_mu;  // serialises API calls that use the stream
+  std::set<zmc_plan *> split_plans;  // plans that hold scratch for split chunks (api_mu)
 
   // pinned staging for host <-> device copies of the blocking calls
   void *stage = nullptr;
@@ -130,6 +132,15 @@ zmc_status ensure_stage(zmc_ctx *ctx, size_t bytes);
 unsigned family_grid(const zmc_ctx *ctx, int family, uint64_t items, int unroll = 1);
 unsigned grid_for(const zmc_ctx *ctx, int family, unsigned block, unsigned bps, uint64_t items,
                   int unroll = 1);
+// Device memory for a table from the context's arena, taking back the plans' split
+// scratch when there is no room otherwise (under api_mu).
+void *arena_take(zmc_ctx *ctx, size_t bytes);
+// Chunks that are handed out by accumulation blocks (LaunchHdr::split).
+constexpr size_t kPartBytes = 32 * sizeof(float2);  // the lane summaries of one block
+constexpr uint64_t kSplitBytes = 8u << 20;          // at most, per family
+uint32_t split_chunks(uint64_t items, bool alike, uint64_t resident_warps, uint32_t quints);
+uint64_t launch_units(uint64_t items, uint32_t split, uint32_t quints);
+unsigned spread_block(unsigned block, uint64_t units, int sms);
 std::string tune_key(const zmc_ctx *ctx, int family, int dim, uint32_t quints, int unroll);
 void tune_cache_load(zmc_ctx *ctx);
 void tune_cache_store(zmc_ctx *ctx, const std::string &key, const TuneChoice &c);

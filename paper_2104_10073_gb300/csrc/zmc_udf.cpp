@@ -210,7 +210,7 @@ struct ArenaBlocks {
   zmc_ctx *ctx;
   std::vector<void *> held;
   void *get(size_t bytes) {
-    void *p = ctx->arena.alloc(bytes);
+    void *p = arena_take(ctx, bytes);
     if (p) held.push_back(p);
     return p;
   }
@@ -272,6 +272,10 @@ zmc_status udf_run(zmc_ctx *ctx, const zmc_udf *udf, const UdfRow *rows, size_t 
   auto *d_out = static_cast<zmc_result *>(ab.get(n * sizeof(zmc_result)));
   auto *d_ent = static_cast<Entry *>(ab.get(ent_b));
   auto *d_mrg = static_cast<const FnDev **>(ab.get(mrg_b));
+  const uint64_t resident = static_cast<uint64_t>(ctx->sms) * udf->max_blocks * 8;
+  bool alike = true;
+  for (size_t i = 1; i < n; ++i) alike = alike && tab[i].variant == tab[0].variant;
+  uint32_t split = split_chunks(total, alike, resident, ctx->quints_per_lane);
   auto *d_hdr = static_cast<LaunchHdr *>(ab.get(sizeof(LaunchHdr)));
   auto *d_p = static_cast<double *>(p_b ? ab.get(p_b) : nullptr);
   if (!d_fns || !d_rec || !d_out || !d_ent || !d_mrg || !d_hdr || (p_b && !d_p))
@@ -316,6 +320,18 @@ zmc_status udf_run(zmc_ctx *ctx, const zmc_udf *udf, const UdfRow *rows, size_t 
     item += (rows[i].n_samples + chunk - 1) / chunk;
   }
   std::memset(hdr, 0, sizeof *hdr);
+  // without room for their scratch, all chunks stay whole
+  float2 *d_part = nullptr;
+  if (split) {
+    d_part = static_cast<float2 *>(
+        ctx->arena.alloc(split * chunk_blocks(ctx->quints_per_lane) * kPartBytes));
+    if (d_part)
+      ab.held.push_back(d_part);
+    else
+      split = 0;
+  }
+  hdr->split[0] = split;
+  hdr->part[0] = d_part;
   hdr->item_end[0] = item;
   hdr->n_entries = static_cast<uint32_t>(n);
   hdr->n_merge = static_cast<uint32_t>(n);
@@ -329,15 +345,18 @@ zmc_status udf_run(zmc_ctx *ctx, const zmc_udf *udf, const UdfRow *rows, size_t 
   if (e == cudaSuccess && p_b) e = cudaMemcpyAsync(d_p, ps, p_b, cudaMemcpyHostToDevice, str);
   if (e == cudaSuccess) {
     // persistent grid: the kernel's occupancy, no more warps than work items
-    const uint64_t want = (item + 7) / 8;
+    const uint64_t units = launch_units(item, split, ctx->quints_per_lane);
+    const unsigned block = spread_block(256, units, ctx->sms);
+    const uint64_t want = (units + block / 32 - 1) / (block / 32);
     const uint64_t cap = static_cast<uint64_t>(ctx->sms) * udf->max_blocks;
     const unsigned grid = static_cast<unsigned>(std::max<uint64_t>(1, std::min(want, cap)));
     const Entry *a0 = d_ent;
     LaunchHdr *a1 = d_hdr;
     void *args[] = {&a0, &a1};
-    e = cudaLaunchKernel(reinterpret_cast<const void *>(udf->k_batched), dim3(grid), dim3(256),
+    e = cudaLaunchKernel(reinterpret_cast<const void *>(udf->k_batched), dim3(grid), dim3(block),
                          args, 0, str);
   }
+  if (e == cudaSuccess) e = launch_combine(d_ent, d_hdr, split, ctx->sms, str);
   if (e == cudaSuccess) {
     const unsigned mg = static_cast<unsigned>(
         std::min<uint64_t>((n + 7) / 8, static_cast<uint64_t>(ctx->sms) * 16));
@@ -404,11 +423,11 @@ zmc_status zmc_udf_create_multi(const char *const *sources, const uint32_t *dims
     const std::string v = "variant_code(ZMC_USER, " + std::to_string(dims[k]) + ", " +
                           std::to_string(k) + ")";
     const std::string targs = "<ZMC_USER, " + std::to_string(dims[k]) + ", " + std::to_string(k) + ">";
-    item_cases += "    case " + v + ": run_item" + targs + "(fn, chunk, Q, lane); break;\n";
+    item_cases += "    case " + v + ": run_item" + targs + "(fn, chunk, Q, lane, span); break;\n";
     eval_cases += "    case " + v + ": eval_range" + targs + "(fn, s_begin, count, out); break;\n";
   }
   prog += "__device__ void udf_dispatch_item(const FnDev *fn, uint64_t chunk, uint32_t Q, "
-          "uint32_t lane) {\n  switch (fn->variant) {\n" + item_cases +
+          "uint32_t lane, const Span span) {\n  switch (fn->variant) {\n" + item_cases +
           "    default: break;\n  }\n}\n"
           "__device__ void udf_dispatch_eval(const FnDev *fn, uint64_t s_begin, uint32_t count, "
           "float *out) {\n  switch (fn->variant) {\n" + eval_cases +

@@ -82,13 +82,14 @@ struct Eval<ZMC_USER, D, G> {
 #endif
 
 // the (dimension, function) switch, generated after this file
-__device__ void udf_dispatch_item(const FnDev *fn, uint64_t chunk, uint32_t Q, uint32_t lane);
+__device__ void udf_dispatch_item(const FnDev *fn, uint64_t chunk, uint32_t Q, uint32_t lane,
+                                  const Span span);
 __device__ void udf_dispatch_eval(const FnDev *fn, uint64_t s_begin, uint32_t count, float *out);
 
 template <>
 __device__ void dispatch_item<ZMC_USER>(const FnDev *fn, uint64_t chunk, uint32_t Q,
-                                        uint32_t lane) {
-  udf_dispatch_item(fn, chunk, Q, lane);
+                                        uint32_t lane, const Span span) {
+  udf_dispatch_item(fn, chunk, Q, lane, span);
 }
 
 template <>
