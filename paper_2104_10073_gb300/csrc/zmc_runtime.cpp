@@ -448,6 +448,20 @@ zmc_status ensure_stage(zmc_ctx *ctx, size_t bytes) {
   return ZMC_OK;
 }
 
+cudaError_t upload_parts(const UploadPart *parts, size_t n, const char *stage, cudaStream_t stream) {
+  cudaError_t e = cudaSuccess;
+  for (size_t k = 0; k < n && e == cudaSuccess;) {
+    const UploadPart &first = parts[k];
+    size_t bytes = first.bytes;
+    for (++k; k < n && static_cast<char *>(parts[k].to) - static_cast<char *>(first.to) ==
+                           static_cast<ptrdiff_t>(parts[k].from - first.from);
+         ++k)
+      bytes = parts[k].from - first.from + parts[k].bytes;
+    e = cudaMemcpyAsync(first.to, stage + first.from, bytes, cudaMemcpyHostToDevice, stream);
+  }
+  return e;
+}
+
 unsigned grid_for(const zmc_ctx *ctx, int family, unsigned block, unsigned bps, uint64_t items,
                   int unroll) {
   const unsigned warps_per_block = block / 32;
@@ -553,6 +567,7 @@ struct zmc_plan {
   FnDev *d_fns = nullptr;
   float2 *d_rec = nullptr;
   zmc_result *d_out = nullptr;
+  zmc_result *h_out = nullptr;  // keep = false: the results in the context's staging
   Entry *d_entries = nullptr;
   LaunchHdr *d_hdr = nullptr;
   const FnDev **d_merge = nullptr;
@@ -730,7 +745,7 @@ zmc_status plan_build(zmc_ctx *ctx, const zmc_desc *desc, size_t n, zmc_plan **o
                       const uint64_t *s_begin = nullptr, const uint64_t *s_end = nullptr,
                       const PlanChoice *force = nullptr, bool keep = true);
 void plan_free(zmc_plan *plan);
-zmc_status plan_enqueue(zmc_plan *plan, uint32_t stages);
+zmc_status plan_enqueue(zmc_plan *plan, uint32_t stages, bool fresh = false);
 
 // The key of a table's shape class for the chunk tuner: the GPU, the families
 // present with their dominant dimension and kernels' registers, and the
@@ -933,9 +948,9 @@ zmc_status choose_chunk(zmc_ctx *ctx, const zmc_desc *desc, size_t n, PlanChoice
 
 // ranges: optional [s_begin[i], s_end[i]) sample ranges (moments output).
 // force: a fixed chunk length and unroll, no autotuning (trial plans).
-// keep = false: the plan goes before the call returns, and the caller's next use of
-// the staging buffer is stream-ordered after the upload (a device-to-host copy of
-// results), so the host need not wait for the upload here.
+// keep = false: the plan goes before the call returns: it has no plain form, its
+// results land in the pinned staging, and the host, which waits for those, need not
+// wait for the upload here.
 zmc_status plan_build(zmc_ctx *ctx, const zmc_desc *desc, size_t n, zmc_plan **out,
                       const uint64_t *s_begin, const uint64_t *s_end, const PlanChoice *force,
                       bool keep) {
@@ -947,18 +962,21 @@ zmc_status plan_build(zmc_ctx *ctx, const zmc_desc *desc, size_t n, zmc_plan **o
   plan->ranged = s_begin != nullptr;
   std::vector<FnDev> fns(n);
   std::vector<uint64_t> len(n);
-  plan->plain.resize(n);
-  plan->volume.resize(n);
+  if (keep) {  // the plain form's tables
+    plan->plain.resize(n);
+    plan->volume.resize(n);
+  }
   // per-descriptor validation and FP64 precompute, in parallel for large tables;
   // the first failing row is redone on this thread for its message
   std::vector<uint8_t> ok(n, 1);
   host_parallel_for(n, 64, [&](size_t b, size_t e) {
     for (size_t i = b; i < e; ++i)
-      ok[i] = precompute(desc[i], &fns[i], &plan->plain[i], &plan->volume[i]) == ZMC_OK;
+      ok[i] = precompute(desc[i], &fns[i], keep ? &plan->plain[i] : nullptr,
+                         keep ? &plan->volume[i] : nullptr) == ZMC_OK;
   });
   for (size_t i = 0; i < n; ++i) {
     if (!ok[i]) {
-      const zmc_status st = precompute(desc[i], &fns[i], &plan->plain[i], &plan->volume[i]);
+      const zmc_status st = precompute(desc[i], &fns[i], nullptr, nullptr);
       return set_error(st, "descriptor %zu: %s", i, zmc_last_error(nullptr));
     }
     len[i] = desc[i].n_samples;
@@ -1001,9 +1019,10 @@ zmc_status plan_build(zmc_ctx *ctx, const zmc_desc *desc, size_t n, zmc_plan **o
   const size_t fn_bytes = n * sizeof(FnDev);
   const size_t ent_bytes = n * sizeof(Entry);
   const size_t mrg_bytes = n * sizeof(FnDev *);
-  plan->d_fns = static_cast<FnDev *>(plan->alloc(fn_bytes));
   plan->d_rec = static_cast<float2 *>(plan->alloc(total * sizeof(float2)));
-  plan->d_out = static_cast<zmc_result *>(plan->alloc(n * sizeof(zmc_result)));
+  if (keep) plan->d_out = static_cast<zmc_result *>(plan->alloc(n * sizeof(zmc_result)));
+  // the uploaded tables one after the other, so that they are usually adjacent
+  plan->d_fns = static_cast<FnDev *>(plan->alloc(fn_bytes));
   plan->d_entries = static_cast<Entry *>(plan->alloc(ent_bytes));
   plan->d_merge = static_cast<const FnDev **>(plan->alloc(mrg_bytes));
   // chunks of each family and how many of them are split
@@ -1025,16 +1044,28 @@ zmc_status plan_build(zmc_ctx *ctx, const zmc_desc *desc, size_t n, zmc_plan **o
     n_split += split[f];
   }
   plan->d_hdr = static_cast<LaunchHdr *>(plan->alloc(sizeof(LaunchHdr)));
-  if (!plan->d_fns || !plan->d_rec || !plan->d_out || !plan->d_entries || !plan->d_merge ||
-      !plan->d_hdr) {
+  if (!plan->d_fns || !plan->d_rec || (keep && !plan->d_out) || !plan->d_entries ||
+      !plan->d_merge || !plan->d_hdr) {
     plan->release_all();
     return set_error(ZMC_ENOMEM, "plan needs %.1f MB of device memory; arena has %.1f MB free",
                      (fn_bytes + total * 8.0 + n * 64.0) / 1e6,
                      ctx->arena.largest_free() / 1e6);
   }
+  // pinned staging: the tables at the arena's granularity, then the results of a
+  // plan that goes before the call returns, which the merge writes straight to the
+  // host (no copy back)
+  const size_t o_ent = round256(fn_bytes), o_mrg = o_ent + round256(ent_bytes),
+               o_hdr = o_mrg + round256(mrg_bytes), o_res = o_hdr + round256(sizeof(LaunchHdr));
+  zmc_status st = ensure_stage(ctx, o_res + (keep ? 0 : n * sizeof(zmc_result)));
+  if (st != ZMC_OK) {
+    plan->release_all();
+    return st;
+  }
+  char *s = static_cast<char *>(ctx->stage);
+  if (!keep) plan->h_out = reinterpret_cast<zmc_result *>(s + o_res);
   for (size_t i = 0; i < n; ++i) {
     fns[i].rec = plan->d_rec + rec_off[i];
-    fns[i].out = plan->d_out + i;
+    fns[i].out = (keep ? plan->d_out : plan->h_out) + i;
   }
   // item order: by family, then variant, then table order
   std::vector<uint32_t> order(n);
@@ -1110,29 +1141,17 @@ zmc_status plan_build(zmc_ctx *ctx, const zmc_desc *desc, size_t n, zmc_plan **o
   std::vector<const FnDev *> merge(n);
   for (size_t i = 0; i < n; ++i) merge[i] = plan->d_fns + i;
 
-  const size_t stage = fn_bytes + ent_bytes + mrg_bytes + sizeof(LaunchHdr);
-  zmc_status st = ensure_stage(ctx, stage);
-  if (st != ZMC_OK) {
-    plan->release_all();
-    return st;
-  }
-  // the staging buffer is reused by the next call, so the copies are waited for
-  // (unless the caller's next use of it is stream-ordered: wait_upload)
-  char *s = static_cast<char *>(ctx->stage);
   std::memcpy(s, fns.data(), fn_bytes);
-  std::memcpy(s + fn_bytes, ents.data(), ent_bytes);
-  std::memcpy(s + fn_bytes + ent_bytes, merge.data(), mrg_bytes);
-  std::memcpy(s + fn_bytes + ent_bytes + mrg_bytes, &h, sizeof h);
+  std::memcpy(s + o_ent, ents.data(), ent_bytes);
+  std::memcpy(s + o_mrg, merge.data(), mrg_bytes);
+  std::memcpy(s + o_hdr, &h, sizeof h);
   cudaStream_t str = ctx->stream;
-  cudaError_t e = cudaMemcpyAsync(plan->d_fns, s, fn_bytes, cudaMemcpyHostToDevice, str);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(plan->d_entries, s + fn_bytes, ent_bytes, cudaMemcpyHostToDevice, str);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(plan->d_merge, s + fn_bytes + ent_bytes, mrg_bytes,
-                        cudaMemcpyHostToDevice, str);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(plan->d_hdr, s + fn_bytes + ent_bytes + mrg_bytes, sizeof h,
-                        cudaMemcpyHostToDevice, str);
+  const UploadPart parts[] = {{plan->d_fns, 0, fn_bytes},
+                              {plan->d_entries, o_ent, ent_bytes},
+                              {plan->d_merge, o_mrg, mrg_bytes},
+                              {plan->d_hdr, o_hdr, sizeof h}};
+  cudaError_t e = upload_parts(parts, 4, s, str);
+  // keep = false: nothing writes the staging's tables before the caller has waited
   if (e == cudaSuccess && keep) e = cudaStreamSynchronize(str);
   if (e != cudaSuccess) {
     plan->release_all();
@@ -1149,11 +1168,13 @@ zmc_status plan_build(zmc_ctx *ctx, const zmc_desc *desc, size_t n, zmc_plan **o
   return ZMC_OK;
 }
 
-zmc_status plan_enqueue(zmc_plan *plan, uint32_t stages) {
+// fresh: the header has just been uploaded and its counters are zero.
+zmc_status plan_enqueue(zmc_plan *plan, uint32_t stages, bool fresh) {
   zmc_ctx *ctx = plan->ctx;
   cudaStream_t str = ctx->stream;
   if (stages & ZMC_STAGE_SAMPLE) {
-    ZMC_CUDA(ctx, cudaMemsetAsync(plan->d_hdr, 0, sizeof(plan->d_hdr->counter), str));
+    if (!fresh)
+      ZMC_CUDA(ctx, cudaMemsetAsync(plan->d_hdr, 0, sizeof(plan->d_hdr->counter), str));
     bool present[4];
     for (int f = 0; f < 4; ++f) present[f] = plan->fam_items[f] > 0;
     ZMC_CUDA(ctx, launch_families(ctx->fork, plan->d_entries, plan->d_hdr, plan->grid,
@@ -1180,6 +1201,19 @@ zmc_status plan_results_to(zmc_plan *plan, zmc_result *out) {
   ZMC_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
   std::memcpy(out, ctx->stage, bytes);
   return ZMC_OK;
+}
+
+// One pass of a plan that was built with keep = false, its results to `out`; the
+// plan goes.
+zmc_status plan_once(zmc_plan *plan, zmc_result *out) {
+  zmc_ctx *ctx = plan->ctx;
+  zmc_status st = plan_enqueue(plan, ZMC_STAGE_ALL, true);
+  const cudaError_t e = cudaStreamSynchronize(ctx->stream);
+  if (st == ZMC_OK && e != cudaSuccess) st = ctx_cuda_fail(ctx, e, "results");
+  if (st == ZMC_OK) std::memcpy(out, plan->h_out, plan->n * sizeof(zmc_result));
+  plan->release_all();
+  delete plan;
+  return st;
 }
 
 void plan_free(zmc_plan *plan) {
@@ -1474,13 +1508,9 @@ zmc_status zmc_integrate(zmc_ctx *ctx, const zmc_desc *desc, size_t n, zmc_resul
   if (!out) return set_error(ZMC_EINVAL, "null output");
   std::lock_guard<std::recursive_mutex> g(ctx->api_mu);
   zmc_plan *plan = nullptr;
-  // the results copy below is the next use of the staging buffer, stream-ordered
   st = plan_build(ctx, desc, n, &plan, nullptr, nullptr, nullptr, false);
   if (st != ZMC_OK) return st;
-  st = plan_enqueue(plan, ZMC_STAGE_ALL);
-  if (st == ZMC_OK) st = plan_results_to(plan, out);
-  plan_free(plan);
-  return st;
+  return plan_once(plan, out);
 }
 
 zmc_status zmc_integrate_plain(zmc_ctx *ctx, const zmc_desc *desc, size_t n, zmc_result *out) {
@@ -1507,10 +1537,7 @@ zmc_status zmc_integrate_moments(zmc_ctx *ctx, const zmc_desc *desc, const uint6
   zmc_plan *plan = nullptr;
   st = plan_build(ctx, desc, n, &plan, s_begin, s_end, nullptr, false);
   if (st != ZMC_OK) return st;
-  st = plan_enqueue(plan, ZMC_STAGE_ALL);
-  if (st == ZMC_OK) st = plan_results_to(plan, reinterpret_cast<zmc_result *>(out));
-  plan_free(plan);
-  return st;
+  return plan_once(plan, reinterpret_cast<zmc_result *>(out));
 }
 
 zmc_status zmc_integrate_functional(zmc_ctx *ctx, const zmc_desc *base, const uint32_t *slots,
@@ -1544,10 +1571,7 @@ zmc_status zmc_integrate_functional(zmc_ctx *ctx, const zmc_desc *base, const ui
   zmc_plan *plan = nullptr;
   st = plan_build(ctx, table.data(), n_points, &plan, nullptr, nullptr, nullptr, false);
   if (st != ZMC_OK) return st;
-  st = plan_enqueue(plan, ZMC_STAGE_ALL);
-  if (st == ZMC_OK) st = plan_results_to(plan, out);
-  plan_free(plan);
-  return st;
+  return plan_once(plan, out);
 }
 
 zmc_status zmc_philox4x32_10(zmc_ctx *ctx, const uint32_t *ctr, const uint32_t *key,

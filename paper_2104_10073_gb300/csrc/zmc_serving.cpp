@@ -129,8 +129,6 @@ struct ServingState {
 
 namespace {
 
-size_t round256(size_t b) { return (b + 255) & ~static_cast<size_t>(255); }
-
 void free_job_device(ServingState *S, ServJob &j) {
   if (j.dblock) {
     S->ctx->arena.release(j.dblock);

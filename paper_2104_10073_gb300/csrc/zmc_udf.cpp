@@ -114,8 +114,6 @@ void put_f32(uint32_t *w, double v) {
 
 void put_f64(uint32_t *w, double v) { std::memcpy(w, &v, 8); }
 
-size_t round256(size_t b) { return (b + 255) & ~static_cast<size_t>(255); }
-
 // FnDev of one user integrand (validated).  For ZMC_UDF_F64 the address of its
 // FP64 parameters is filled in by udf_run.
 zmc_status udf_fn(const zmc_udf *u, const UdfRow &d, size_t i, FnDev *fn) {
@@ -267,9 +265,9 @@ zmc_status udf_run(zmc_ctx *ctx, const zmc_udf *udf, const UdfRow *rows, size_t 
   ArenaBlocks ab{ctx, {}};
   const size_t fn_b = n * sizeof(FnDev), ent_b = n * sizeof(Entry), mrg_b = n * sizeof(FnDev *),
                p_b = params.size() * ZMC_NPARAM * sizeof(double);
-  auto *d_fns = static_cast<FnDev *>(ab.get(fn_b));
   auto *d_rec = static_cast<float2 *>(ab.get(total * sizeof(float2)));
-  auto *d_out = static_cast<zmc_result *>(ab.get(n * sizeof(zmc_result)));
+  // the uploaded tables one after the other, so that they are usually adjacent
+  auto *d_fns = static_cast<FnDev *>(ab.get(fn_b));
   auto *d_ent = static_cast<Entry *>(ab.get(ent_b));
   auto *d_mrg = static_cast<const FnDev **>(ab.get(mrg_b));
   const uint64_t resident = static_cast<uint64_t>(ctx->sms) * udf->max_blocks * 8;
@@ -278,15 +276,16 @@ zmc_status udf_run(zmc_ctx *ctx, const zmc_udf *udf, const UdfRow *rows, size_t 
   uint32_t split = split_chunks(total, alike, resident, ctx->quints_per_lane);
   auto *d_hdr = static_cast<LaunchHdr *>(ab.get(sizeof(LaunchHdr)));
   auto *d_p = static_cast<double *>(p_b ? ab.get(p_b) : nullptr);
-  if (!d_fns || !d_rec || !d_out || !d_ent || !d_mrg || !d_hdr || (p_b && !d_p))
+  if (!d_fns || !d_rec || !d_ent || !d_mrg || !d_hdr || (p_b && !d_p))
     return set_error(ZMC_ENOMEM, "udf call needs %.1f MB of device memory",
                      (fn_b + total * 8.0 + n * 64.0 + p_b) / 1e6);
 
-  // host tables in the pinned staging buffer: fns | entries | merge list | hdr | params
+  // host tables in the pinned staging buffer: fns | entries | merge list | hdr | params,
+  // then the results, which the merge writes there
   const size_t o_ent = round256(fn_b), o_mrg = o_ent + round256(ent_b),
                o_hdr = o_mrg + round256(mrg_b), o_p = o_hdr + round256(sizeof(LaunchHdr)),
-               o_end = o_p + round256(p_b);
-  st = ensure_stage(ctx, std::max(o_end, n * sizeof(zmc_result)));
+               o_res = o_p + round256(p_b);
+  st = ensure_stage(ctx, o_res + n * sizeof(zmc_result));
   if (st != ZMC_OK) return st;
   char *s = static_cast<char *>(ctx->stage);
   auto *fns = reinterpret_cast<FnDev *>(s);
@@ -294,13 +293,14 @@ zmc_status udf_run(zmc_ctx *ctx, const zmc_udf *udf, const UdfRow *rows, size_t 
   auto *mrg = reinterpret_cast<const FnDev **>(s + o_mrg);
   auto *hdr = reinterpret_cast<LaunchHdr *>(s + o_hdr);
   auto *ps = reinterpret_cast<double *>(s + o_p);
+  auto *res = reinterpret_cast<zmc_result *>(s + o_res);
   for (size_t q = 0; q < params.size(); ++q)
     std::memcpy(ps + q * ZMC_NPARAM, params[q], ZMC_NPARAM * sizeof(double));
   for (size_t i = 0; i < n; ++i) {
     fns[i] = tab[i];
     if (f64) set_param_address(&fns[i], d_p + static_cast<size_t>(prow[i]) * ZMC_NPARAM);
     fns[i].rec = d_rec + rec_off[i];
-    fns[i].out = d_out + i;
+    fns[i].out = res + i;
     mrg[i] = d_fns + i;
   }
   // the work list runs the rows grouped by variant (dimension and user function),
@@ -338,11 +338,12 @@ zmc_status udf_run(zmc_ctx *ctx, const zmc_udf *udf, const UdfRow *rows, size_t 
   hdr->quints_per_lane = ctx->quints_per_lane;
 
   cudaStream_t str = ctx->stream;
-  e = cudaMemcpyAsync(d_fns, fns, fn_b, cudaMemcpyHostToDevice, str);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(d_ent, ents, ent_b, cudaMemcpyHostToDevice, str);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(d_mrg, mrg, mrg_b, cudaMemcpyHostToDevice, str);
-  if (e == cudaSuccess) e = cudaMemcpyAsync(d_hdr, hdr, sizeof *hdr, cudaMemcpyHostToDevice, str);
-  if (e == cudaSuccess && p_b) e = cudaMemcpyAsync(d_p, ps, p_b, cudaMemcpyHostToDevice, str);
+  const UploadPart parts[] = {{d_fns, 0, fn_b},
+                              {d_ent, o_ent, ent_b},
+                              {d_mrg, o_mrg, mrg_b},
+                              {d_hdr, o_hdr, sizeof *hdr},
+                              {d_p, o_p, p_b}};
+  e = upload_parts(parts, p_b ? 5 : 4, s, str);
   if (e == cudaSuccess) {
     // persistent grid: the kernel's occupancy, no more warps than work items
     const uint64_t units = launch_units(item, split, ctx->quints_per_lane);
@@ -362,11 +363,11 @@ zmc_status udf_run(zmc_ctx *ctx, const zmc_udf *udf, const UdfRow *rows, size_t 
         std::min<uint64_t>((n + 7) / 8, static_cast<uint64_t>(ctx->sms) * 16));
     e = launch_merge(d_mrg, d_hdr, mg, str);
   }
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(s, d_out, n * sizeof(zmc_result), cudaMemcpyDeviceToHost, str);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(str);
+  // also after an error: the arena blocks go back below
+  const cudaError_t sync = cudaStreamSynchronize(str);
+  if (e == cudaSuccess) e = sync;
   if (e != cudaSuccess) return ctx_cuda_fail(ctx, e, "udf integrate");
-  std::memcpy(out, s, n * sizeof(zmc_result));
+  std::memcpy(out, res, n * sizeof(zmc_result));
   return ZMC_OK;
 }
 
