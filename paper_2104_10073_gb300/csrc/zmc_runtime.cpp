@@ -434,6 +434,17 @@ zmc_status precompute(const zmc_desc &d, FnDev *fn, PlainFn *plain, double *volu
   return ZMC_OK;
 }
 
+// Rows per range of a parallel loop over a table's precompute: ranges of ~10 us (a
+// product polynomial of degree >= 2 takes its factors' roots, ~2.5 us each on one
+// core; any other row ~0.3 us), the whole table when it is not worth waking a worker.
+size_t precompute_grain(const zmc_desc *desc, size_t n) {
+  double us = 0.0;
+  for (size_t i = 0; i < n; ++i)
+    us += desc[i].family == ZMC_POLY && desc[i].deg >= 2 ? 2.5 * std::min(desc[i].dim, 7u) : 0.3;
+  if (us < 40.0) return n;
+  return std::max<size_t>(1, std::min<size_t>(64, static_cast<size_t>(10.0 * n / us)));
+}
+
 zmc_status ensure_stage(zmc_ctx *ctx, size_t bytes) {
   if (ctx->stage_bytes >= bytes) return ZMC_OK;
   if (ctx->stage) {
@@ -969,7 +980,7 @@ zmc_status plan_build(zmc_ctx *ctx, const zmc_desc *desc, size_t n, zmc_plan **o
   // per-descriptor validation and FP64 precompute, in parallel for large tables;
   // the first failing row is redone on this thread for its message
   std::vector<uint8_t> ok(n, 1);
-  host_parallel_for(n, 64, [&](size_t b, size_t e) {
+  host_parallel_for(n, precompute_grain(desc, n), [&](size_t b, size_t e) {
     for (size_t i = b; i < e; ++i)
       ok[i] = precompute(desc[i], &fns[i], keep ? &plan->plain[i] : nullptr,
                          keep ? &plan->volume[i] : nullptr) == ZMC_OK;
@@ -1070,11 +1081,13 @@ zmc_status plan_build(zmc_ctx *ctx, const zmc_desc *desc, size_t n, zmc_plan **o
   // item order: by family, then variant, then table order
   std::vector<uint32_t> order(n);
   std::iota(order.begin(), order.end(), 0u);
-  std::stable_sort(order.begin(), order.end(), [&](uint32_t a, uint32_t b) {
+  const auto before = [&](uint32_t a, uint32_t b) {
     const uint32_t fa = desc[a].family, fb = desc[b].family;
     if (fa != fb) return fa < fb;
     return fns[a].variant < fns[b].variant;
-  });
+  };
+  if (!std::is_sorted(order.begin(), order.end(), before))
+    std::stable_sort(order.begin(), order.end(), before);
   std::vector<Entry> ents(n);
   LaunchHdr &h = plan->h_hdr;
   std::memset(&h, 0, sizeof h);
@@ -1290,7 +1303,7 @@ size_t zmc_desc_size(void) { return sizeof(zmc_desc); }
 zmc_status zmc_validate(const zmc_desc *desc, size_t n, size_t *bad_index) {
   if (!desc && n) return set_error(ZMC_EINVAL, "null descriptor table");
   std::vector<uint8_t> ok(n, 1);
-  host_parallel_for(n, 64, [&](size_t b, size_t e) {
+  host_parallel_for(n, precompute_grain(desc, n), [&](size_t b, size_t e) {
     FnDev fn;
     for (size_t i = b; i < e; ++i) ok[i] = precompute(desc[i], &fn, nullptr, nullptr) == ZMC_OK;
   });

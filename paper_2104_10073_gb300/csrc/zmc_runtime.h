@@ -46,6 +46,9 @@ class Arena {
 // Derived device form of one descriptor (validation + FP64 precompute).
 zmc_status precompute(const zmc_desc &d, FnDev *fn, PlainFn *plain, double *volume);
 
+// Rows per range for host_parallel_for over precompute.
+size_t precompute_grain(const zmc_desc *desc, size_t n);
+
 // Launch-shape choice for the per-family persistent kernels.
 struct LaunchShape {
   unsigned block = 256;

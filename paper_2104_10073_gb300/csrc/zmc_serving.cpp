@@ -708,7 +708,7 @@ zmc_status submit_job(zmc_ctx *ctx, const zmc_desc *desc, const zmc_moments *fro
   j->next_chunk.assign(n, 0);
   const uint64_t chunk = chunk_samples_of(ctx->quints_per_lane);
   std::vector<uint8_t> ok(n, 1);
-  host_parallel_for(n, 64, [&](size_t b, size_t e) {
+  host_parallel_for(n, precompute_grain(desc, n), [&](size_t b, size_t e) {
     for (size_t i = b; i < e; ++i) ok[i] = precompute(desc[i], &j->fns[i], nullptr, nullptr) == ZMC_OK;
   });
   for (size_t i = 0; i < n; ++i) {

@@ -16,6 +16,7 @@
 #include <dlfcn.h>
 
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstring>
 #include <mutex>
@@ -244,42 +245,17 @@ zmc_status udf_run(zmc_ctx *ctx, const zmc_udf *udf, const UdfRow *rows, size_t 
 
   const bool f64 = udf->precision == ZMC_UDF_F64;
   const uint64_t chunk = chunk_samples_of(ctx->quints_per_lane);
-  std::vector<FnDev> tab(n);
-  std::vector<uint64_t> rec_off(n);
-  std::vector<uint32_t> prow(n);        // FP64: index of the row's parameter block
-  std::vector<const double *> params;   // distinct parameter arrays, in first-use order
-  uint64_t total = 0;
-  for (size_t i = 0; i < n; ++i) {
-    st = udf_fn(udf, rows[i], i, &tab[i]);  // validates
-    if (st != ZMC_OK) return st;
-    rec_off[i] = total;
-    total += (rows[i].n_samples + chunk - 1) / chunk;
-    if (f64) {
-      if (params.empty() || params.back() != rows[i].p) {
-        if (params.size() >= (1u << 24)) return set_error(ZMC_EINVAL, "too many parameter rows");
-        params.push_back(rows[i].p);
-      }
-      prow[i] = static_cast<uint32_t>(params.size() - 1);
+  std::vector<uint32_t> prow(f64 ? n : 0);  // FP64: index of the row's parameter block
+  std::vector<const double *> params;       // distinct parameter arrays, in first-use order
+  for (size_t i = 0; f64 && i < n; ++i) {
+    if (params.empty() || params.back() != rows[i].p) {
+      if (params.size() >= (1u << 24)) return set_error(ZMC_EINVAL, "too many parameter rows");
+      params.push_back(rows[i].p);
     }
+    prow[i] = static_cast<uint32_t>(params.size() - 1);
   }
-  ArenaBlocks ab{ctx, {}};
   const size_t fn_b = n * sizeof(FnDev), ent_b = n * sizeof(Entry), mrg_b = n * sizeof(FnDev *),
                p_b = params.size() * ZMC_NPARAM * sizeof(double);
-  auto *d_rec = static_cast<float2 *>(ab.get(total * sizeof(float2)));
-  // the uploaded tables one after the other, so that they are usually adjacent
-  auto *d_fns = static_cast<FnDev *>(ab.get(fn_b));
-  auto *d_ent = static_cast<Entry *>(ab.get(ent_b));
-  auto *d_mrg = static_cast<const FnDev **>(ab.get(mrg_b));
-  const uint64_t resident = static_cast<uint64_t>(ctx->sms) * udf->max_blocks * 8;
-  bool alike = true;
-  for (size_t i = 1; i < n; ++i) alike = alike && tab[i].variant == tab[0].variant;
-  uint32_t split = split_chunks(total, alike, resident, ctx->quints_per_lane);
-  auto *d_hdr = static_cast<LaunchHdr *>(ab.get(sizeof(LaunchHdr)));
-  auto *d_p = static_cast<double *>(p_b ? ab.get(p_b) : nullptr);
-  if (!d_fns || !d_rec || !d_ent || !d_mrg || !d_hdr || (p_b && !d_p))
-    return set_error(ZMC_ENOMEM, "udf call needs %.1f MB of device memory",
-                     (fn_b + total * 8.0 + n * 64.0 + p_b) / 1e6);
-
   // host tables in the pinned staging buffer: fns | entries | merge list | hdr | params,
   // then the results, which the merge writes there
   const size_t o_ent = round256(fn_b), o_mrg = o_ent + round256(ent_b),
@@ -294,14 +270,48 @@ zmc_status udf_run(zmc_ctx *ctx, const zmc_udf *udf, const UdfRow *rows, size_t 
   auto *hdr = reinterpret_cast<LaunchHdr *>(s + o_hdr);
   auto *ps = reinterpret_cast<double *>(s + o_p);
   auto *res = reinterpret_cast<zmc_result *>(s + o_res);
+  // validation and constants straight into the staging, in ranges of ~20 us; the
+  // first failing row is redone on this thread for its message
+  std::atomic<size_t> bad{n};
+  host_parallel_for(n, n < 512 ? n : 128, [&](size_t b, size_t e) {
+    for (size_t i = b; i < e; ++i) {
+      if (udf_fn(udf, rows[i], i, &fns[i]) == ZMC_OK) continue;
+      size_t first = bad.load();
+      while (i < first && !bad.compare_exchange_weak(first, i)) {
+      }
+      return;
+    }
+  });
+  if (bad.load() < n) return udf_fn(udf, rows[bad.load()], bad.load(), &fns[bad.load()]);
+  uint64_t total = 0;
+  bool alike = true, sorted = true;
+  for (size_t i = 0; i < n; ++i) {
+    total += (rows[i].n_samples + chunk - 1) / chunk;
+    alike = alike && fns[i].variant == fns[0].variant;
+    sorted = sorted && (i == 0 || fns[i - 1].variant <= fns[i].variant);
+  }
+  ArenaBlocks ab{ctx, {}};
+  auto *d_rec = static_cast<float2 *>(ab.get(total * sizeof(float2)));
+  // the uploaded tables one after the other, so that they are usually adjacent
+  auto *d_fns = static_cast<FnDev *>(ab.get(fn_b));
+  auto *d_ent = static_cast<Entry *>(ab.get(ent_b));
+  auto *d_mrg = static_cast<const FnDev **>(ab.get(mrg_b));
+  const uint64_t resident = static_cast<uint64_t>(ctx->sms) * udf->max_blocks * 8;
+  uint32_t split = split_chunks(total, alike, resident, ctx->quints_per_lane);
+  auto *d_hdr = static_cast<LaunchHdr *>(ab.get(sizeof(LaunchHdr)));
+  auto *d_p = static_cast<double *>(p_b ? ab.get(p_b) : nullptr);
+  if (!d_fns || !d_rec || !d_ent || !d_mrg || !d_hdr || (p_b && !d_p))
+    return set_error(ZMC_ENOMEM, "udf call needs %.1f MB of device memory",
+                     (fn_b + total * 8.0 + n * 64.0 + p_b) / 1e6);
   for (size_t q = 0; q < params.size(); ++q)
     std::memcpy(ps + q * ZMC_NPARAM, params[q], ZMC_NPARAM * sizeof(double));
+  uint64_t rec = 0;
   for (size_t i = 0; i < n; ++i) {
-    fns[i] = tab[i];
     if (f64) set_param_address(&fns[i], d_p + static_cast<size_t>(prow[i]) * ZMC_NPARAM);
-    fns[i].rec = d_rec + rec_off[i];
+    fns[i].rec = d_rec + rec;
     fns[i].out = res + i;
     mrg[i] = d_fns + i;
+    rec += (rows[i].n_samples + chunk - 1) / chunk;
   }
   // the work list runs the rows grouped by variant (dimension and user function),
   // so that consecutive work items, which co-resident warps take, use the same
@@ -309,8 +319,9 @@ zmc_status udf_run(zmc_ctx *ctx, const zmc_udf *udf, const UdfRow *rows, size_t 
   // changes no result
   std::vector<uint32_t> order(n);
   for (size_t i = 0; i < n; ++i) order[i] = static_cast<uint32_t>(i);
-  std::stable_sort(order.begin(), order.end(),
-                   [&](uint32_t a, uint32_t b) { return tab[a].variant < tab[b].variant; });
+  if (!sorted)
+    std::stable_sort(order.begin(), order.end(),
+                     [&](uint32_t a, uint32_t b) { return fns[a].variant < fns[b].variant; });
   uint64_t item = 0;
   for (size_t k = 0; k < n; ++k) {
     const uint32_t i = order[k];
