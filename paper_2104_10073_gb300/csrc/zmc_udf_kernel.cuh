@@ -73,8 +73,13 @@ struct Eval<ZMC_USER, D, G> {
     double x[D];
 #pragma unroll
     for (int i = 0; i < D; ++i) {
-      const double u = static_cast<double>(r[i] & 0x7FFFFFu) * 0x1p-23;
-      x[i] = fma(wd[i], u, lo[i]);
+      // 1 + u from its bits by three integer operations, then an exact subtraction: one
+      // FP64 operation where the conversion and its scaling took two; the FP64 pipe
+      // (2 lanes an SM) is what bounds this kernel (100 rows of
+      // 10^5 samples, cos and sin of a 4-D phase: 1088 -> 1004 us)
+      const double v = __hiloint2double(static_cast<int>(0x3FF00000u | ((r[i] >> 3) & 0xFFFFFu)),
+                                        static_cast<int>(r[i] << 29));
+      x[i] = fma(wd[i], v - 1.0, lo[i]);
     }
     return static_cast<float>(S * UserFn<G>::f(x, p));
   }
