@@ -549,7 +549,7 @@ struct HdrSlot {
 // chunks last every warp is busy, but a launch of few chunks, and the end of a
 // launch whose chunks differ in length, would leave most of the chip idle for up to
 // a chunk's time (60 .. 190 us at Q = 104).  A block's lane summaries go to the
-// launch's scratch, and zmc_combine_kernel makes the chunks' records of them.
+// launch's scratch, and zmc_finish_kernel makes the chunks' records of them.
 // (Counting a chunk's blocks and combining them here, in the warp that completes the
 // count, kept so much state alive over the chunk's body that whole chunks of the
 // polynomial kernel slowed down by 3%; drawing the next item before the body, to

@@ -171,11 +171,12 @@ constexpr int kMaxUnroll = 2;
 // cudaError_t; an unknown family or unroll gives cudaErrorInvalidValue.
 cudaError_t launch_batched(int family, const Entry *entries, LaunchHdr *hdr, unsigned grid,
                            unsigned block, cudaStream_t stream, int unroll = 1);
-// The records of a launch's split chunks (`chunks` of them over the families).
-cudaError_t launch_combine(const Entry *entries, const LaunchHdr *hdr, uint64_t chunks, int sms,
-                           cudaStream_t stream);
-cudaError_t launch_merge(const FnDev *const *fns, const LaunchHdr *hdr, unsigned grid,
-                         cudaStream_t stream);
+cudaError_t launch_merge(const FnDev *const *fns, LaunchHdr *hdr, unsigned grid,
+                         cudaStream_t stream, bool reset = false);
+// The records of a launch's split chunks and the merge of its rows (n_entries rows,
+// one entry each); warps: split chunks + rows; left: n_entries zeros.
+cudaError_t launch_finish(const Entry *entries, LaunchHdr *hdr, uint32_t *left, uint64_t warps,
+                          int sms, cudaStream_t stream);
 cudaError_t launch_plain(const PlainFn &fn, double *block_rec, unsigned grid,
                          cudaStream_t stream);
 cudaError_t launch_plain_merge(const PlainJob *jobs, uint32_t n, cudaStream_t stream);

@@ -67,28 +67,6 @@ __device__ __forceinline__ void combine_blocks(const FnDev *__restrict__ fn, uin
   if (lane == 0) fn->rec[chunk] = make_float2(mean, m2);
 }
 
-// One warp per split chunk of a launch (LaunchHdr::split), of any family: a few
-// loads and ~13 dependent merge steps each, so it is bound by latency; 304 blocks
-// hold all of a launch's warps at once.
-__global__ void __launch_bounds__(256) zmc_combine_kernel(const Entry *__restrict__ entries,
-                                                          const LaunchHdr *__restrict__ hdr) {
-  const uint32_t lane = threadIdx.x & 31u;
-  const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
-  const uint32_t Q = hdr->quints_per_lane;
-  uint32_t w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  for (int f = 0; f < 4; ++f) {
-    const uint32_t split = hdr->split[f];
-    for (; w < split; w += nwarps) {
-      const uint64_t item = hdr->item_end[f] - split + w;
-      const Entry en = entries[find_entry(entries, hdr->n_entries, item, lane)];
-      const uint64_t chunk = en.chunk_begin + (item - en.item_begin);
-      combine_blocks(en.fn, chunk, samples_of(en.fn, chunk, Q), Q, lane,
-                     hdr->part[f] + static_cast<size_t>(w) * 32u * chunk_blocks(Q));
-    }
-    w -= split;  // the next family's chunks go on with the next warp
-  }
-}
-
 // ---------------------------------------------------------------- FP64 merge
 // One warp per integrand.  With chunk summaries (n_c, m_c, M2_c):
 //   mean = sum_c n_c m_c / N,  M2 = sum_c [M2_c + n_c (m_c - mean)^2]
@@ -97,59 +75,129 @@ __global__ void __launch_bounds__(256) zmc_combine_kernel(const Entry *__restric
 // of earlier samples of the stream (prior_n > 0) are combined in last with the
 // pairwise update, n = n_a + n_b, mean = mean_a + d n_b / n,
 // M2 = M2_a + M2_b + d^2 n_a n_b / n, d = mean_b - mean_a.
+// A chain of loads and FP64 steps, so bound by latency: the first kHeld records of a
+// lane are loaded at once and held for the second pass (most rows have no more).
+__device__ __forceinline__ void merge_row(const FnDev *__restrict__ fn, uint64_t chunk_samples,
+                                          uint32_t lane) {
+  constexpr uint32_t kHeld = 4;
+  const uint64_t N = fn->n_samples;
+  const uint64_t C = (N + chunk_samples - 1) / chunk_samples;
+  const float2 *rec = fn->rec;  // perhaps written by this launch: read past the L1
+  const auto weight = [&](uint64_t c) {
+    const uint64_t left = N - c * chunk_samples;
+    return static_cast<double>(left < chunk_samples ? left : chunk_samples);
+  };
+  float2 held[kHeld];
+#pragma unroll
+  for (uint32_t i = 0; i < kHeld; ++i)
+    if (lane + 32 * i < C) held[i] = __ldcg(rec + lane + 32 * i);
+  double s = 0.0;
+#pragma unroll
+  for (uint32_t i = 0; i < kHeld; ++i)
+    if (lane + 32 * i < C) s = fma(weight(lane + 32 * i), static_cast<double>(held[i].x), s);
+  for (uint64_t c = lane + 32 * kHeld; c < C; c += 32)
+    s = fma(weight(c), static_cast<double>(__ldcg(rec + c).x), s);
+  const double mean = N ? warp_sum_f64(s) / static_cast<double>(N) : 0.0;
+  double m = 0.0;
+  const auto spread = [&](uint64_t c, float2 rc) {
+    const double dm = static_cast<double>(rc.x) - mean;
+    m += fma(weight(c) * dm, dm, static_cast<double>(rc.y));
+  };
+#pragma unroll
+  for (uint32_t i = 0; i < kHeld; ++i)
+    if (lane + 32 * i < C) spread(lane + 32 * i, held[i]);
+  for (uint64_t c = lane + 32 * kHeld; c < C; c += 32) spread(c, __ldcg(rec + c));
+  const double inv = fn->inv_scale;
+  double mu = mean * inv;
+  double m2 = fmax(warp_sum_f64(m), 0.0) * inv * inv;
+  uint64_t n_all = N;
+  if (fn->prior_n > 0) {
+    const double na = static_cast<double>(fn->prior_n), nb = static_cast<double>(N);
+    const double nab = na + nb;
+    const double d = mu - fn->prior_mean;
+    mu = fn->prior_mean + d * (nb / nab);
+    m2 = fn->prior_m2 + m2 + d * d * (na * nb / nab);
+    n_all = fn->prior_n + N;
+  }
+  if (lane == 0) {
+    const double nd = static_cast<double>(n_all);
+    zmc_result res;
+    if (fn->out_mode == 0) {
+      res.estimate = fn->volume * mu;
+      res.stderr_ = fn->volume * sqrt(m2 / (nd * (nd - 1.0)));
+    } else {  // zmc_moments: unscaled mean and M2 of f over the samples
+      res.estimate = mu;
+      res.stderr_ = m2;
+    }
+    res.n = n_all;
+    res.status = ZMC_OK;
+    res.reserved = 0;
+    *fn->out = res;
+  }
+}
+
+// reset: the launch's counters go back to zero for its next run (the sampling
+// kernels that drew from them have ended), which saves a memset per run.
 __global__ void __launch_bounds__(256) zmc_merge_kernel(const FnDev *const *__restrict__ fns,
-                                                        const LaunchHdr *__restrict__ hdr) {
+                                                        LaunchHdr *__restrict__ hdr, bool reset) {
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
   const uint32_t nm = hdr->n_merge;
   const uint64_t chunk_samples = chunk_samples_of(hdr->quints_per_lane);
-  for (uint32_t k = warp; k < nm; k += nwarps) {
-    const FnDev *fn = fns[k];
-    const uint64_t N = fn->n_samples;
-    const uint64_t C = (N + chunk_samples - 1) / chunk_samples;
-    const float2 *rec = fn->rec;
-    double s = 0.0;
-    for (uint64_t c = lane; c < C; c += 32) {
-      const uint64_t left = N - c * chunk_samples;
-      const double nc = static_cast<double>(left < chunk_samples ? left : chunk_samples);
-      s = fma(nc, static_cast<double>(rec[c].x), s);
-    }
-    const double mean = N ? warp_sum_f64(s) / static_cast<double>(N) : 0.0;
-    double m = 0.0;
-    for (uint64_t c = lane; c < C; c += 32) {
-      const uint64_t left = N - c * chunk_samples;
-      const double nc = static_cast<double>(left < chunk_samples ? left : chunk_samples);
-      const float2 rc = rec[c];
-      const double dm = static_cast<double>(rc.x) - mean;
-      m += fma(nc * dm, dm, static_cast<double>(rc.y));
-    }
-    const double inv = fn->inv_scale;
-    double mu = mean * inv;
-    double m2 = fmax(warp_sum_f64(m), 0.0) * inv * inv;
-    uint64_t n_all = N;
-    if (fn->prior_n > 0) {
-      const double na = static_cast<double>(fn->prior_n), nb = static_cast<double>(N);
-      const double nab = na + nb;
-      const double d = mu - fn->prior_mean;
-      mu = fn->prior_mean + d * (nb / nab);
-      m2 = fn->prior_m2 + m2 + d * d * (na * nb / nab);
-      n_all = fn->prior_n + N;
-    }
-    if (lane == 0) {
-      const double nd = static_cast<double>(n_all);
-      zmc_result res;
-      if (fn->out_mode == 0) {
-        res.estimate = fn->volume * mu;
-        res.stderr_ = fn->volume * sqrt(m2 / (nd * (nd - 1.0)));
-      } else {  // zmc_moments: unscaled mean and M2 of f over the samples
-        res.estimate = mu;
-        res.stderr_ = m2;
-      }
-      res.n = n_all;
-      res.status = ZMC_OK;
-      res.reserved = 0;
-      *fn->out = res;
+  if (reset && warp == 0 && lane < 4) hdr->counter[lane] = 0;
+  for (uint32_t k = warp; k < nm; k += nwarps) merge_row(fns[k], chunk_samples, lane);
+}
+
+// The merge of a launch with split chunks, whose entries are its rows in some order:
+// one warp per split chunk makes its record, and the warp that completes a row's
+// count of split chunks merges the row; one warp per row without any merges it at
+// once.  One kernel less than records and merge apart (~4 us of a small call).
+// left: a count per entry, zero before the first run; it wraps to zero by itself.
+__global__ void __launch_bounds__(256) zmc_finish_kernel(const Entry *__restrict__ entries,
+                                                         LaunchHdr *__restrict__ hdr,
+                                                         uint32_t *__restrict__ left) {
+  const uint32_t lane = threadIdx.x & 31u;
+  const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
+  const uint32_t Q = hdr->quints_per_lane;
+  const uint32_t ne = hdr->n_entries;
+  uint32_t total = 0;
+  for (int f = 0; f < 4; ++f) total += hdr->split[f];
+  uint32_t w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (w == 0 && lane < 4) hdr->counter[lane] = 0;
+  for (; w < total + ne; w += nwarps) {
+    if (w < total) {
+      int f = 0;
+      uint32_t t = w;
+      for (; t >= hdr->split[f]; ++f) t -= hdr->split[f];
+      const uint64_t split0 = hdr->item_end[f] - hdr->split[f];  // the family's first split item
+      const uint32_t e = find_entry(entries, ne, split0 + t, lane);
+      const Entry en = entries[e];
+      const uint64_t chunk = en.chunk_begin + (split0 + t - en.item_begin);
+      combine_blocks(en.fn, chunk, samples_of(en.fn, chunk, Q), Q, lane,
+                     hdr->part[f] + static_cast<size_t>(t) * 32u * chunk_blocks(Q));
+      const uint64_t next = e + 1 < ne ? entries[e + 1].item_begin : hdr->item_end[f];
+      const uint64_t end = next < hdr->item_end[f] ? next : hdr->item_end[f];
+      const uint32_t last =
+          static_cast<uint32_t>(end - (en.item_begin > split0 ? en.item_begin : split0)) - 1;
+      uint32_t before = 0;
+      if (lane == 0)  // after this lane's record
+        asm volatile("atom.acq_rel.gpu.global.inc.u32 %0, [%1], %2;"
+                     : "=r"(before)
+                     : "l"(left + e), "r"(last)
+                     : "memory");
+      before = __shfl_sync(kFullMask, before, 0);
+      if (before != last) continue;
+      __threadfence();
+      merge_row(en.fn, chunk_samples_of(Q), lane);
+    } else {
+      const uint32_t e = w - total;
+      const Entry en = entries[e];
+      const uint32_t family = (en.fn->variant >> 4) & 0xFu;
+      const uint32_t f = family < 4 ? family : 0;  // HdrSlot
+      const uint64_t next = e + 1 < ne ? entries[e + 1].item_begin : hdr->item_end[f];
+      const uint64_t end = next < hdr->item_end[f] ? next : hdr->item_end[f];
+      if (end <= hdr->item_end[f] - hdr->split[f]) merge_row(en.fn, chunk_samples_of(Q), lane);
     }
   }
 }
@@ -209,17 +257,16 @@ cudaError_t launch_batched(int family, const Entry *entries, LaunchHdr *hdr, uns
   return ops ? ops->launch_batched(entries, hdr, grid, block, stream) : cudaErrorInvalidValue;
 }
 
-cudaError_t launch_merge(const FnDev *const *fns, const LaunchHdr *hdr, unsigned grid,
-                         cudaStream_t stream) {
-  zmc_merge_kernel<<<grid, 256, 0, stream>>>(fns, hdr);
+cudaError_t launch_merge(const FnDev *const *fns, LaunchHdr *hdr, unsigned grid,
+                         cudaStream_t stream, bool reset) {
+  zmc_merge_kernel<<<grid, 256, 0, stream>>>(fns, hdr, reset);
   return cudaGetLastError();
 }
 
-cudaError_t launch_combine(const Entry *entries, const LaunchHdr *hdr, uint64_t chunks, int sms,
-                           cudaStream_t stream) {
-  if (chunks == 0) return cudaSuccess;
-  const uint64_t blocks = std::min<uint64_t>((chunks + 7) / 8, 2ull * static_cast<unsigned>(sms));
-  zmc_combine_kernel<<<static_cast<unsigned>(blocks), 256, 0, stream>>>(entries, hdr);
+cudaError_t launch_finish(const Entry *entries, LaunchHdr *hdr, uint32_t *left, uint64_t warps,
+                          int sms, cudaStream_t stream) {
+  const uint64_t blocks = std::min<uint64_t>((warps + 7) / 8, 16ull * static_cast<unsigned>(sms));
+  zmc_finish_kernel<<<static_cast<unsigned>(blocks), 256, 0, stream>>>(entries, hdr, left);
   return cudaGetLastError();
 }
 

@@ -195,7 +195,7 @@ extern "C" zmc_status zmc_integrate_noalloc(const zmc_desc *desc, size_t n, zmc_
   }
   const unsigned mgrid = static_cast<unsigned>(std::min<size_t>((n + 7) / 8, static_cast<size_t>(sms) * 16));
   e = launch_merge(reinterpret_cast<const FnDev *const *>(dbase + off_mrg),
-                   reinterpret_cast<const LaunchHdr *>(dbase + kOffHdr), mgrid, str);
+                   reinterpret_cast<LaunchHdr *>(dbase + kOffHdr), mgrid, str);
   if (e != cudaSuccess) return set_error(ZMC_ECUDA, "merge launch: %s", cudaGetErrorString(e));
   return ZMC_OK;
 }

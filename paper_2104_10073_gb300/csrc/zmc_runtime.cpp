@@ -592,7 +592,9 @@ struct zmc_plan {
   uint64_t n_chunks = 0, n_samples = 0;
   uint64_t fam_items[4] = {0, 0, 0, 0};
   uint64_t fam_units[4] = {0, 0, 0, 0};  // whole chunks and blocks of split ones
-  void *d_part = nullptr;  // lane summaries of the split chunks
+  void *d_part = nullptr;     // lane summaries of the split chunks
+  uint32_t *d_left = nullptr;  // counts of the finish kernel, when chunks may be split
+  bool dirty = false;          // the counters were drawn from and not reset
   bool ranged = false;  // built by zmc_integrate_moments (no plain form)
   uint32_t quints = 0;  // chunk = 160 * quints samples
   unsigned unroll[4] = {1, 1, 1, 1};  // quint-loop unroll of each family kernel
@@ -627,6 +629,13 @@ namespace zmc {
 static void drop_splits(zmc_ctx *ctx) {
   bool ok = true;
   for (zmc_plan *p : ctx->split_plans) {
+    if (p->dirty) {  // sampled, not merged yet: the records are still to be made
+      uint64_t warps = p->n;
+      for (uint32_t k : p->h_hdr.split) warps += k;
+      ok = ok && launch_finish(p->d_entries, p->d_hdr, p->d_left, warps, ctx->sms, ctx->stream) ==
+                     cudaSuccess;
+      p->dirty = false;
+    }
     std::memset(p->h_hdr.split, 0, sizeof p->h_hdr.split);
     ok = ok && cudaMemcpyAsync(p->d_hdr, &p->h_hdr, sizeof p->h_hdr, cudaMemcpyHostToDevice,
                                ctx->stream) == cudaSuccess;
@@ -756,7 +765,8 @@ zmc_status plan_build(zmc_ctx *ctx, const zmc_desc *desc, size_t n, zmc_plan **o
                       const uint64_t *s_begin = nullptr, const uint64_t *s_end = nullptr,
                       const PlanChoice *force = nullptr, bool keep = true);
 void plan_free(zmc_plan *plan);
-zmc_status plan_enqueue(zmc_plan *plan, uint32_t stages, bool fresh = false);
+zmc_status plan_reset(zmc_plan *plan);
+zmc_status plan_enqueue(zmc_plan *plan, uint32_t stages);
 
 // The key of a table's shape class for the chunk tuner: the GPU, the families
 // present with their dominant dimension and kernels' registers, and the
@@ -1054,7 +1064,8 @@ zmc_status plan_build(zmc_ctx *ctx, const zmc_desc *desc, size_t n, zmc_plan **o
                             static_cast<uint64_t>(ctx->sms) * 8 * std::max(bps, 1), plan->quints);
     n_split += split[f];
   }
-  plan->d_hdr = static_cast<LaunchHdr *>(plan->alloc(sizeof(LaunchHdr)));
+  const size_t hdr_bytes = sizeof(LaunchHdr) + (n_split ? n * sizeof(uint32_t) : 0);
+  plan->d_hdr = static_cast<LaunchHdr *>(plan->alloc(hdr_bytes));
   if (!plan->d_fns || !plan->d_rec || (keep && !plan->d_out) || !plan->d_entries ||
       !plan->d_merge || !plan->d_hdr) {
     plan->release_all();
@@ -1066,7 +1077,7 @@ zmc_status plan_build(zmc_ctx *ctx, const zmc_desc *desc, size_t n, zmc_plan **o
   // plan that goes before the call returns, which the merge writes straight to the
   // host (no copy back)
   const size_t o_ent = round256(fn_bytes), o_mrg = o_ent + round256(ent_bytes),
-               o_hdr = o_mrg + round256(mrg_bytes), o_res = o_hdr + round256(sizeof(LaunchHdr));
+               o_hdr = o_mrg + round256(mrg_bytes), o_res = o_hdr + round256(hdr_bytes);
   zmc_status st = ensure_stage(ctx, o_res + (keep ? 0 : n * sizeof(zmc_result)));
   if (st != ZMC_OK) {
     plan->release_all();
@@ -1125,6 +1136,7 @@ zmc_status plan_build(zmc_ctx *ctx, const zmc_desc *desc, size_t n, zmc_plan **o
     plan->d_part = ctx->arena.alloc(n_split * nb * kPartBytes);
   if (plan->d_part) {
     ctx->split_plans.insert(plan.get());
+    plan->d_left = reinterpret_cast<uint32_t *>(plan->d_hdr + 1);
     auto *part = static_cast<float2 *>(plan->d_part);
     for (int f = 0; f < 4; ++f) {
       h.split[f] = split[f];
@@ -1158,11 +1170,12 @@ zmc_status plan_build(zmc_ctx *ctx, const zmc_desc *desc, size_t n, zmc_plan **o
   std::memcpy(s + o_ent, ents.data(), ent_bytes);
   std::memcpy(s + o_mrg, merge.data(), mrg_bytes);
   std::memcpy(s + o_hdr, &h, sizeof h);
+  std::memset(s + o_hdr + sizeof h, 0, hdr_bytes - sizeof h);
   cudaStream_t str = ctx->stream;
   const UploadPart parts[] = {{plan->d_fns, 0, fn_bytes},
                               {plan->d_entries, o_ent, ent_bytes},
                               {plan->d_merge, o_mrg, mrg_bytes},
-                              {plan->d_hdr, o_hdr, sizeof h}};
+                              {plan->d_hdr, o_hdr, hdr_bytes}};
   cudaError_t e = upload_parts(parts, 4, s, str);
   // keep = false: nothing writes the staging's tables before the caller has waited
   if (e == cudaSuccess && keep) e = cudaStreamSynchronize(str);
@@ -1181,25 +1194,39 @@ zmc_status plan_build(zmc_ctx *ctx, const zmc_desc *desc, size_t n, zmc_plan **o
   return ZMC_OK;
 }
 
-// fresh: the header has just been uploaded and its counters are zero.
-zmc_status plan_enqueue(zmc_plan *plan, uint32_t stages, bool fresh) {
+// The counters are zero after the upload and after each merge; a sampling stage run
+// by itself leaves them drawn from.
+zmc_status plan_reset(zmc_plan *plan) {
+  if (!plan->dirty) return ZMC_OK;
+  ZMC_CUDA(plan->ctx, cudaMemsetAsync(plan->d_hdr, 0, sizeof(plan->d_hdr->counter),
+                                      plan->ctx->stream));
+  plan->dirty = false;
+  return ZMC_OK;
+}
+
+zmc_status plan_enqueue(zmc_plan *plan, uint32_t stages) {
   zmc_ctx *ctx = plan->ctx;
   cudaStream_t str = ctx->stream;
   if (stages & ZMC_STAGE_SAMPLE) {
-    if (!fresh)
-      ZMC_CUDA(ctx, cudaMemsetAsync(plan->d_hdr, 0, sizeof(plan->d_hdr->counter), str));
+    const zmc_status st = plan_reset(plan);
+    if (st != ZMC_OK) return st;
+    plan->dirty = true;
     bool present[4];
     for (int f = 0; f < 4; ++f) present[f] = plan->fam_items[f] > 0;
     ZMC_CUDA(ctx, launch_families(ctx->fork, plan->d_entries, plan->d_hdr, plan->grid,
                                   plan->block, present, str, plan->unroll));
-    uint64_t split = 0;
-    for (uint32_t s : plan->h_hdr.split) split += s;
-    ZMC_CUDA(ctx, launch_combine(plan->d_entries, plan->d_hdr, split, ctx->sms, str));
   }
   if (stages & ZMC_STAGE_MERGE) {
-    const unsigned grid = static_cast<unsigned>(
-        std::min<size_t>((plan->n + 7) / 8, static_cast<size_t>(ctx->sms) * 16));
-    ZMC_CUDA(ctx, launch_merge(plan->d_merge, plan->d_hdr, grid, str));
+    if (plan->d_left) {  // also after the scratch went: then every row merges at once
+      uint64_t warps = plan->n;
+      for (uint32_t k : plan->h_hdr.split) warps += k;
+      ZMC_CUDA(ctx, launch_finish(plan->d_entries, plan->d_hdr, plan->d_left, warps, ctx->sms, str));
+    } else {
+      const unsigned grid = static_cast<unsigned>(
+          std::min<size_t>((plan->n + 7) / 8, static_cast<size_t>(ctx->sms) * 16));
+      ZMC_CUDA(ctx, launch_merge(plan->d_merge, plan->d_hdr, grid, str, true));
+    }
+    plan->dirty = false;
   }
   return ZMC_OK;
 }
@@ -1220,7 +1247,7 @@ zmc_status plan_results_to(zmc_plan *plan, zmc_result *out) {
 // plan goes.
 zmc_status plan_once(zmc_plan *plan, zmc_result *out) {
   zmc_ctx *ctx = plan->ctx;
-  zmc_status st = plan_enqueue(plan, ZMC_STAGE_ALL, true);
+  zmc_status st = plan_enqueue(plan, ZMC_STAGE_ALL);
   const cudaError_t e = cudaStreamSynchronize(ctx->stream);
   if (st == ZMC_OK && e != cudaSuccess) st = ctx_cuda_fail(ctx, e, "results");
   if (st == ZMC_OK) std::memcpy(out, plan->h_out, plan->n * sizeof(zmc_result));
@@ -1445,6 +1472,8 @@ zmc_status zmc_plan_run(zmc_plan *plan, uint32_t stages) {
     return set_error(ZMC_EINVAL, "stages must be a non-empty subset of ZMC_STAGE_ALL");
   std::lock_guard<std::recursive_mutex> g(ctx->api_mu);
   if (stages != ZMC_STAGE_ALL) return plan_enqueue(plan, stages);
+  st = plan_reset(plan);  // outside the graph, which is captured with clean counters
+  if (st != ZMC_OK) return st;
   if (!plan->graph) {
     cudaGraph_t graph = nullptr;
     ZMC_CUDA(ctx, cudaStreamBeginCapture(ctx->stream, cudaStreamCaptureModeThreadLocal));

@@ -245,6 +245,7 @@ zmc_status udf_run(zmc_ctx *ctx, const zmc_udf *udf, const UdfRow *rows, size_t 
 
   const bool f64 = udf->precision == ZMC_UDF_F64;
   const uint64_t chunk = chunk_samples_of(ctx->quints_per_lane);
+  const size_t hdr_b = sizeof(LaunchHdr) + n * sizeof(uint32_t);  // + the finish kernel's counts
   std::vector<uint32_t> prow(f64 ? n : 0);  // FP64: index of the row's parameter block
   std::vector<const double *> params;       // distinct parameter arrays, in first-use order
   for (size_t i = 0; f64 && i < n; ++i) {
@@ -259,7 +260,7 @@ zmc_status udf_run(zmc_ctx *ctx, const zmc_udf *udf, const UdfRow *rows, size_t 
   // host tables in the pinned staging buffer: fns | entries | merge list | hdr | params,
   // then the results, which the merge writes there
   const size_t o_ent = round256(fn_b), o_mrg = o_ent + round256(ent_b),
-               o_hdr = o_mrg + round256(mrg_b), o_p = o_hdr + round256(sizeof(LaunchHdr)),
+               o_hdr = o_mrg + round256(mrg_b), o_p = o_hdr + round256(hdr_b),
                o_res = o_p + round256(p_b);
   st = ensure_stage(ctx, o_res + n * sizeof(zmc_result));
   if (st != ZMC_OK) return st;
@@ -298,7 +299,7 @@ zmc_status udf_run(zmc_ctx *ctx, const zmc_udf *udf, const UdfRow *rows, size_t 
   auto *d_mrg = static_cast<const FnDev **>(ab.get(mrg_b));
   const uint64_t resident = static_cast<uint64_t>(ctx->sms) * udf->max_blocks * 8;
   uint32_t split = split_chunks(total, alike, resident, ctx->quints_per_lane);
-  auto *d_hdr = static_cast<LaunchHdr *>(ab.get(sizeof(LaunchHdr)));
+  auto *d_hdr = static_cast<LaunchHdr *>(ab.get(hdr_b));
   auto *d_p = static_cast<double *>(p_b ? ab.get(p_b) : nullptr);
   if (!d_fns || !d_rec || !d_ent || !d_mrg || !d_hdr || (p_b && !d_p))
     return set_error(ZMC_ENOMEM, "udf call needs %.1f MB of device memory",
@@ -330,7 +331,7 @@ zmc_status udf_run(zmc_ctx *ctx, const zmc_udf *udf, const UdfRow *rows, size_t 
     ents[k].chunk_begin = 0;
     item += (rows[i].n_samples + chunk - 1) / chunk;
   }
-  std::memset(hdr, 0, sizeof *hdr);
+  std::memset(hdr, 0, hdr_b);
   // without room for their scratch, all chunks stay whole
   float2 *d_part = nullptr;
   if (split) {
@@ -352,7 +353,7 @@ zmc_status udf_run(zmc_ctx *ctx, const zmc_udf *udf, const UdfRow *rows, size_t 
   const UploadPart parts[] = {{d_fns, 0, fn_b},
                               {d_ent, o_ent, ent_b},
                               {d_mrg, o_mrg, mrg_b},
-                              {d_hdr, o_hdr, sizeof *hdr},
+                              {d_hdr, o_hdr, hdr_b},
                               {d_p, o_p, p_b}};
   e = upload_parts(parts, p_b ? 5 : 4, s, str);
   if (e == cudaSuccess) {
@@ -368,8 +369,10 @@ zmc_status udf_run(zmc_ctx *ctx, const zmc_udf *udf, const UdfRow *rows, size_t 
     e = cudaLaunchKernel(reinterpret_cast<const void *>(udf->k_batched), dim3(grid), dim3(block),
                          args, 0, str);
   }
-  if (e == cudaSuccess) e = launch_combine(d_ent, d_hdr, split, ctx->sms, str);
-  if (e == cudaSuccess) {
+  if (e == cudaSuccess && split) {
+    e = launch_finish(d_ent, d_hdr, reinterpret_cast<uint32_t *>(d_hdr + 1), n + split, ctx->sms,
+                      str);
+  } else if (e == cudaSuccess) {
     const unsigned mg = static_cast<unsigned>(
         std::min<uint64_t>((n + 7) / 8, static_cast<uint64_t>(ctx->sms) * 16));
     e = launch_merge(d_mrg, d_hdr, mg, str);

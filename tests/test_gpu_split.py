@@ -59,3 +59,27 @@ def test_scratch_returns_to_the_arena():
         assert np.array_equal(first["stderr"], got["stderr"])
         zmc.zmc_plan_destroy(pa)
         zmc.zmc_plan_destroy(pb)
+
+
+def test_scratch_taken_back_between_the_stages():
+    """A sampling stage whose merge comes after another table took the scratch; and
+    stages repeated by themselves."""
+    rng = np.random.default_rng(4)
+    a = W.random_table(40, rng, families=(W.GAUSS,), dims=(1, 7))
+    a["n_samples"] = 16640 * 15
+    b = W.random_table(3000, rng, n_lo=10, n_hi=20, families=(W.POLY,))
+    with zmc.Context(arena_bytes=2 << 20) as c:
+        want = zmc.zmc_integrate(c.handle, a)
+        pa = zmc.zmc_plan_create(c.handle, a)
+        zmc.zmc_plan_run(pa, zmc.ZMC_STAGE_SAMPLE)
+        zmc.zmc_plan_run(pa, zmc.ZMC_STAGE_SAMPLE)
+        pb = zmc.zmc_plan_create(c.handle, b)
+        for stages in ((zmc.ZMC_STAGE_MERGE,), (zmc.ZMC_STAGE_MERGE,), (zmc.ZMC_STAGE_ALL,),
+                       (zmc.ZMC_STAGE_SAMPLE, zmc.ZMC_STAGE_ALL)):
+            for stage in stages:
+                zmc.zmc_plan_run(pa, stage)
+            got = zmc.zmc_plan_results(pa, len(a))
+            assert np.array_equal(got["estimate"], want["estimate"]), stages
+            assert np.array_equal(got["stderr"], want["stderr"]), stages
+        zmc.zmc_plan_destroy(pa)
+        zmc.zmc_plan_destroy(pb)
