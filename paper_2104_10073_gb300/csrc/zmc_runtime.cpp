@@ -1089,13 +1089,21 @@ zmc_status plan_build(zmc_ctx *ctx, const zmc_desc *desc, size_t n, zmc_plan **o
     fns[i].rec = plan->d_rec + rec_off[i];
     fns[i].out = (keep ? plan->d_out : plan->h_out) + i;
   }
-  // item order: by family, then variant, then table order
+  // item order: by family, then variant, then table order; in a launch that hands out
+  // every chunk by blocks, high dimensions first, so that a family's last blocks are
+  // its shortest (a 1-D block takes a tenth of a 7-D one's time: 64 mixed rows 291 ->
+  // 272 us).  Larger launches gain nothing from it (300 mixed rows 1117 -> 1130 us).
+  bool blocks_only = true;
+  for (int f = 0; f < 4; ++f) blocks_only = blocks_only && split[f] == fam_chunks[f];
+  const auto rank = [&](uint32_t variant) {
+    return blocks_only ? ((15u - (variant & 15u)) << 16) | variant : variant;
+  };
   std::vector<uint32_t> order(n);
   std::iota(order.begin(), order.end(), 0u);
   const auto before = [&](uint32_t a, uint32_t b) {
     const uint32_t fa = desc[a].family, fb = desc[b].family;
     if (fa != fb) return fa < fb;
-    return fns[a].variant < fns[b].variant;
+    return rank(fns[a].variant) < rank(fns[b].variant);
   };
   if (!std::is_sorted(order.begin(), order.end(), before))
     std::stable_sort(order.begin(), order.end(), before);
