@@ -13,6 +13,8 @@
 //                        fixed order: mean, M2, estimate = V mean,
 //                        stderr = V sqrt(M2 / (N (N-1))) (Fig. 1 caption: an estimate
 //                        with its spread).
+//   zmc_finish_kernel    for a launch whose last chunks were handed out by
+//                        accumulation blocks: their records, then the same merge.
 //   zmc_plain_fp64_kernel  (zmc_plain.cu) the plain form, one launch per integrand.
 //   zmc_philox_rate_kernel  the generator alone (its throughput: the ceiling of
 //                        any sampling kernel, which draws d / 5 blocks per sample).
