@@ -39,8 +39,8 @@ struct Loop {
 };
 
 // The caller waits for the ranges, not for the workers: with 15 workers to wake and
-// hear from, a loop of 20 us took 60.  It wakes one worker, and each that finds work
-// wakes the next.
+// hear from, a loop of 20 us took 60.  For a few ranges it wakes one worker, and each
+// that finds work wakes the next; a loop of many ranges wakes them all.
 class HostPool {
  public:
   HostPool() {
@@ -62,7 +62,10 @@ class HostPool {
       loop_ = loop;
       ++gen_;
     }
-    cv_.notify_one();
+    if (n / grain >= 2 * workers_.size())
+      cv_.notify_all();
+    else
+      cv_.notify_one();
     if (loop->work()) return;
     std::unique_lock<std::mutex> lk(mu_);
     done_cv_.wait(lk, [&] { return loop->done.load(std::memory_order_acquire) == n; });
