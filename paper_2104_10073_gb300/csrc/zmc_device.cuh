@@ -333,7 +333,7 @@ __device__ __forceinline__ void run_chunk(const FnDev *__restrict__ fn, uint64_t
                                           bool crossing) {
   Eval<FAM, D, G> ev;
   ev.load(fn);
-  const uint32_t key0 = fn->key0, key1 = fn->key1;
+  const RoundKeys rk = make_round_keys(fn->key0, fn->key1);
   const uint32_t sid = fn->stream_id;
   const uint64_t chunk_samples = chunk_samples_of(Q);
   const uint64_t s0 = chunk * chunk_samples;
@@ -342,8 +342,7 @@ __device__ __forceinline__ void run_chunk(const FnDev *__restrict__ fn, uint64_t
   const uint64_t quint0 = (fn->s_off + s0) / kQuint;  // s_off is a multiple of 5
   const uint64_t block0 = quint0 * D;
   const uint32_t base_lo0 = static_cast<uint32_t>(block0) + lane * D;
-  const StreamPrefix sp = make_stream_prefix(make_round_keys(key0, key1), sid,
-                                             static_cast<uint32_t>(block0 >> 32));
+  const StreamPrefix sp = make_stream_prefix(rk, sid, static_cast<uint32_t>(block0 >> 32));
 
   // running (n, mean, M2) of the lane, merged from blocks of kBlockQuints quints
   float n = 0.0f, mean = 0.0f, m2 = 0.0f;
@@ -364,7 +363,7 @@ __device__ __forceinline__ void run_chunk(const FnDev *__restrict__ fn, uint64_t
       if (FAST || !crossing)
         gen_quint_fast<D>(base_lo0 + 32u * D * j, sp, r);
       else
-        gen_quint<D>(quint0 + ql, sid, make_round_keys(key0, key1), r);
+        gen_quint<D>(quint0 + ql, sid, rk, r);
       float f[5];
       eval_quint<D>(ev, r, f);
       if (j == jb) {

@@ -500,8 +500,8 @@ unsigned family_grid(const zmc_ctx *ctx, int family, uint64_t items, int unroll)
 // anyway (4864: 171 either way, 188 split).
 // Chunks that differ in cost (families, dimensions, polynomial degrees) leave a tail
 // of up to the longest chunk's time at the end and a CTA's slowest warp's time at
-// each change of family: one chunk per resident warp fills it (300 mixed rows 1117
-// against 1295 us, 64 mixed rows 295 against 386).
+// each change of family: one chunk per resident warp fills it (300 mixed rows 1107
+// against 1295 us, 64 mixed rows 271 against 386).
 // The lane summaries take 256 bytes a block, at most kSplitBytes a family (5 MB at
 // the default Q = 104).  None for chunks of one block.
 uint32_t split_chunks(uint64_t items, bool alike, uint64_t resident_warps, uint32_t quints) {
