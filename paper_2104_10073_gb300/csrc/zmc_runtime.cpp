@@ -1064,8 +1064,14 @@ zmc_status plan_build(zmc_ctx *ctx, const zmc_desc *desc, size_t n, zmc_plan **o
                             static_cast<uint64_t>(ctx->sms) * 8 * std::max(bps, 1), plan->quints);
     n_split += split[f];
   }
-  const size_t hdr_bytes = sizeof(LaunchHdr) + (n_split ? n * sizeof(uint32_t) : 0);
+  // the header and, after it, the finish kernel's counts; no room for those: no split
+  size_t hdr_bytes = sizeof(LaunchHdr) + (n_split ? n * sizeof(uint32_t) : 0);
   plan->d_hdr = static_cast<LaunchHdr *>(plan->alloc(hdr_bytes));
+  if (!plan->d_hdr && n_split) {
+    n_split = 0;
+    hdr_bytes = sizeof(LaunchHdr);
+    plan->d_hdr = static_cast<LaunchHdr *>(plan->alloc(hdr_bytes));
+  }
   if (!plan->d_fns || !plan->d_rec || (keep && !plan->d_out) || !plan->d_entries ||
       !plan->d_merge || !plan->d_hdr) {
     plan->release_all();

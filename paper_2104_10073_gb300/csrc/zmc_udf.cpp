@@ -245,7 +245,7 @@ zmc_status udf_run(zmc_ctx *ctx, const zmc_udf *udf, const UdfRow *rows, size_t 
 
   const bool f64 = udf->precision == ZMC_UDF_F64;
   const uint64_t chunk = chunk_samples_of(ctx->quints_per_lane);
-  const size_t hdr_b = sizeof(LaunchHdr) + n * sizeof(uint32_t);  // + the finish kernel's counts
+  size_t hdr_b = sizeof(LaunchHdr) + n * sizeof(uint32_t);  // + the finish kernel's counts
   std::vector<uint32_t> prow(f64 ? n : 0);  // FP64: index of the row's parameter block
   std::vector<const double *> params;       // distinct parameter arrays, in first-use order
   for (size_t i = 0; f64 && i < n; ++i) {
@@ -299,7 +299,13 @@ zmc_status udf_run(zmc_ctx *ctx, const zmc_udf *udf, const UdfRow *rows, size_t 
   auto *d_mrg = static_cast<const FnDev **>(ab.get(mrg_b));
   const uint64_t resident = static_cast<uint64_t>(ctx->sms) * udf->max_blocks * 8;
   uint32_t split = split_chunks(total, alike, resident, ctx->quints_per_lane);
+  if (!split) hdr_b = sizeof(LaunchHdr);
   auto *d_hdr = static_cast<LaunchHdr *>(ab.get(hdr_b));
+  if (!d_hdr && split) {  // no room for the counts: no split
+    split = 0;
+    hdr_b = sizeof(LaunchHdr);
+    d_hdr = static_cast<LaunchHdr *>(ab.get(hdr_b));
+  }
   auto *d_p = static_cast<double *>(p_b ? ab.get(p_b) : nullptr);
   if (!d_fns || !d_rec || !d_ent || !d_mrg || !d_hdr || (p_b && !d_p))
     return set_error(ZMC_ENOMEM, "udf call needs %.1f MB of device memory",
