@@ -459,16 +459,21 @@ zmc_status ensure_stage(zmc_ctx *ctx, size_t bytes) {
   return ZMC_OK;
 }
 
+// Joined are parts that follow one another at the arena's granularity on both sides:
+// then the bytes between them are the padding of their own blocks.  (An equal distance
+// on both sides is not enough: in the arena another table may lie in between.)
 cudaError_t upload_parts(const UploadPart *parts, size_t n, const char *stage, cudaStream_t stream) {
+  const auto follows = [&](const UploadPart &a, const UploadPart &b) {
+    return static_cast<char *>(a.to) + round256(a.bytes) == b.to &&
+           a.from + round256(a.bytes) == b.from;
+  };
   cudaError_t e = cudaSuccess;
   for (size_t k = 0; k < n && e == cudaSuccess;) {
     const UploadPart &first = parts[k];
-    size_t bytes = first.bytes;
-    for (++k; k < n && static_cast<char *>(parts[k].to) - static_cast<char *>(first.to) ==
-                           static_cast<ptrdiff_t>(parts[k].from - first.from);
-         ++k)
-      bytes = parts[k].from - first.from + parts[k].bytes;
-    e = cudaMemcpyAsync(first.to, stage + first.from, bytes, cudaMemcpyHostToDevice, stream);
+    for (++k; k < n && follows(parts[k - 1], parts[k]);) ++k;
+    const UploadPart &last = parts[k - 1];
+    e = cudaMemcpyAsync(first.to, stage + first.from, last.from + last.bytes - first.from,
+                        cudaMemcpyHostToDevice, stream);
   }
   return e;
 }

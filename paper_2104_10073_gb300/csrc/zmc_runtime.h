@@ -137,7 +137,8 @@ unsigned grid_for(const zmc_ctx *ctx, int family, unsigned block, unsigned bps, 
                   int unroll = 1);
 constexpr size_t round256(size_t b) { return (b + 255) & ~static_cast<size_t>(255); }
 // Tables in the pinned staging (in order, at 256-byte offsets) to the device: those
-// that lie as in the staging go up in one copy (~2 us of host and of GPU time each).
+// that follow one another there too go up in one copy (~2 us of host and of GPU time
+// each).
 struct UploadPart {
   void *to;
   size_t from, bytes;

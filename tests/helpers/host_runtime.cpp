@@ -1,0 +1,215 @@
+// The host runtime (plans, user calls, arena, staging) on a CUDA that is not there:
+// device memory is host memory, every copy and launch happens at once and is noted.
+// Each scenario prints one line per fact for tests/test_host_runtime.py.
+#include <cstdarg>
+#include <cstdio>
+#include <cstdlib>
+#include <string>
+
+#include "zmc_udf.cpp"  // struct zmc_udf is defined there
+
+// ---------------------------------------------------------------- the CUDA that is not there
+namespace {
+struct Range {
+  uintptr_t begin, end;
+  bool meets(const Range &o) const { return begin < o.end && o.begin < end; }
+};
+std::vector<Range> g_uploads;       // host-to-device copies
+std::vector<std::string> g_events;  // launches and counter resets, in order
+
+void note(const char *fmt, ...) {
+  char buf[256];
+  va_list ap;
+  va_start(ap, fmt);
+  std::vsnprintf(buf, sizeof buf, fmt, ap);
+  va_end(ap);
+  g_events.push_back(buf);
+}
+uint32_t splits(const LaunchHdr *h) { return h->split[0] + h->split[1] + h->split[2] + h->split[3]; }
+}  // namespace
+
+extern "C" {
+cudaError_t cudaGetDeviceCount(int *n) { return *n = 1, cudaSuccess; }
+cudaError_t cudaSetDevice(int) { return cudaSuccess; }
+cudaError_t cudaGetDeviceProperties(cudaDeviceProp *p, int) {
+  std::memset(p, 0, sizeof *p);
+  std::strcpy(p->name, "none");
+  p->multiProcessorCount = 152;
+  return cudaSuccess;
+}
+const char *cudaGetErrorString(cudaError_t) { return "error"; }
+cudaError_t cudaStreamCreateWithFlags(cudaStream_t *s, unsigned) {
+  return *s = reinterpret_cast<cudaStream_t>(std::malloc(1)), cudaSuccess;
+}
+cudaError_t cudaStreamDestroy(cudaStream_t s) { return std::free(s), cudaSuccess; }
+cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned) { return cudaSuccess; }
+cudaError_t cudaEventCreate(cudaEvent_t *e) {
+  return *e = reinterpret_cast<cudaEvent_t>(std::malloc(1)), cudaSuccess;
+}
+cudaError_t cudaEventCreateWithFlags(cudaEvent_t *e, unsigned) { return cudaEventCreate(e); }
+cudaError_t cudaEventDestroy(cudaEvent_t e) { return std::free(e), cudaSuccess; }
+cudaError_t cudaEventRecord(cudaEvent_t, cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaEventSynchronize(cudaEvent_t) { return cudaSuccess; }
+cudaError_t cudaEventElapsedTime(float *ms, cudaEvent_t, cudaEvent_t) { return *ms = 1.0f, cudaSuccess; }
+cudaError_t cudaMalloc(void **p, size_t n) {
+  return *p = std::aligned_alloc(256, (n + 255) & ~size_t{255}), cudaSuccess;
+}
+cudaError_t cudaFree(void *p) { return std::free(p), cudaSuccess; }
+cudaError_t cudaHostAlloc(void **p, size_t n, unsigned) { return cudaMalloc(p, n); }
+cudaError_t cudaFreeHost(void *p) { return std::free(p), cudaSuccess; }
+cudaError_t cudaMemcpyAsync(void *to, const void *from, size_t n, cudaMemcpyKind kind, cudaStream_t) {
+  if (kind == cudaMemcpyHostToDevice)
+    g_uploads.push_back({reinterpret_cast<uintptr_t>(to), reinterpret_cast<uintptr_t>(to) + n});
+  std::memmove(to, from, n);
+  return cudaSuccess;
+}
+cudaError_t cudaMemsetAsync(void *to, int v, size_t n, cudaStream_t) {
+  note("memset");
+  std::memset(to, v, n);
+  return cudaSuccess;
+}
+cudaError_t cudaStreamBeginCapture(cudaStream_t, cudaStreamCaptureMode) { return cudaSuccess; }
+cudaError_t cudaStreamEndCapture(cudaStream_t, cudaGraph_t *g) { return *g = nullptr, cudaSuccess; }
+cudaError_t cudaGraphInstantiate(cudaGraphExec_t *x, cudaGraph_t, unsigned long long) {
+  return *x = reinterpret_cast<cudaGraphExec_t>(std::malloc(1)), cudaSuccess;
+}
+cudaError_t cudaGraphLaunch(cudaGraphExec_t, cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaGraphDestroy(cudaGraph_t) { return cudaSuccess; }
+cudaError_t cudaGraphExecDestroy(cudaGraphExec_t x) { return std::free(x), cudaSuccess; }
+cudaError_t cudaLaunchKernel(const void *, dim3, dim3, void **args, size_t, cudaStream_t) {
+  note("udf split %u", splits(*static_cast<LaunchHdr **>(args[1])));
+  return cudaSuccess;
+}
+cudaError_t cudaLibraryLoadData(cudaLibrary_t *, const void *, cudaJitOption *, void **, unsigned,
+                                cudaLibraryOption *, void **, unsigned) {
+  return cudaErrorNotSupported;
+}
+cudaError_t cudaLibraryUnload(cudaLibrary_t) { return cudaSuccess; }
+cudaError_t cudaLibraryGetKernel(cudaKernel_t *, cudaLibrary_t, const char *) {
+  return cudaErrorNotSupported;
+}
+cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessor(int *n, const void *, int, size_t) {
+  return *n = 2, cudaSuccess;
+}
+}  // extern "C"
+
+zmc_status serving_start(zmc_ctx *) { return ZMC_OK; }
+void serving_stop(zmc_ctx *) {}
+
+namespace zmc {
+cudaError_t launch_batched(int f, const Entry *, LaunchHdr *h, unsigned, unsigned, cudaStream_t, int) {
+  note("batched %d split %u", f, h->split[f]);
+  h->counter[f] = h->item_end[f] - h->item_begin[f];
+  return cudaSuccess;
+}
+cudaError_t launch_merge(const FnDev *const *, LaunchHdr *h, unsigned, cudaStream_t, bool reset) {
+  note("merge");
+  if (reset) std::memset(h->counter, 0, sizeof h->counter);
+  return cudaSuccess;
+}
+cudaError_t launch_finish(const Entry *, LaunchHdr *h, uint32_t *, uint64_t, int, cudaStream_t) {
+  note("finish split %u", splits(h));
+  std::memset(h->counter, 0, sizeof h->counter);
+  return cudaSuccess;
+}
+cudaError_t launch_plain(const PlainFn &, double *, unsigned, cudaStream_t) { return cudaSuccess; }
+cudaError_t launch_plain_merge(const PlainJob *, uint32_t, cudaStream_t) { return cudaSuccess; }
+cudaError_t launch_philox(const uint32_t *, const uint32_t *, uint32_t *, size_t, cudaStream_t) {
+  return cudaSuccess;
+}
+cudaError_t launch_eval(int, const FnDev *, uint64_t, uint32_t, float *, cudaStream_t) {
+  return cudaSuccess;
+}
+cudaError_t launch_philox_rate(uint32_t, unsigned, uint32_t *, cudaStream_t) { return cudaSuccess; }
+int batched_max_blocks_per_sm(int, int, int) { return 2; }
+int batched_regs_per_thread(int, int) { return 128; }
+unsigned plain_grid(const PlainFn &, int) { return 1; }
+}  // namespace zmc
+
+// ---------------------------------------------------------------- scenarios
+namespace {
+
+zmc_ctx *context(size_t bytes, uint32_t quints) {
+  zmc_options o;
+  zmc_default_options(&o);
+  o.mem_budget_bytes = bytes;
+  o.quints_per_lane = quints;
+  zmc_ctx *c = nullptr;
+  if (zmc_create(&o, &c) != ZMC_OK) std::abort();
+  return c;
+}
+
+std::vector<zmc_desc> gauss_rows(size_t n, uint32_t dim, uint64_t samples) {
+  zmc_desc d;
+  std::memset(&d, 0, sizeof d);
+  d.family = ZMC_GAUSS;
+  d.dim = dim;
+  d.n_samples = samples;
+  d.p[0] = 1.0;
+  d.p[1] = 0.1;
+  for (uint32_t k = 0; k < dim; ++k) {
+    d.hi[k] = 1.0;
+    d.p[2 + k] = 0.5;
+  }
+  return std::vector<zmc_desc>(n, d);
+}
+
+zmc_udf *user(uint32_t precision) {
+  auto *u = new zmc_udf;
+  u->dims = {1};
+  u->scales = {1.0};
+  u->precision = precision;
+  u->max_blocks = 2;
+  u->lib = reinterpret_cast<cudaLibrary_t>(1);
+  return u;
+}
+
+zmc_plan *plan(zmc_ctx *c, const std::vector<zmc_desc> &rows) {
+  zmc_plan *p = nullptr;
+  return zmc_plan_create(c, rows.data(), rows.size(), &p) == ZMC_OK ? p : nullptr;
+}
+
+// Parts whose staging slots and device blocks are as far apart, with room in between
+// that is not theirs.
+void upload_gap() {
+  char dev[4096], stage[4096];
+  const UploadPart parts[] = {{dev, 0, 160}, {dev + 2048, 2048, 300}, {dev + 2560, 2560, 10}};
+  upload_parts(parts, 3, stage, nullptr);
+  for (const Range &r : g_uploads)
+    std::printf("%zu %zu\n", r.begin - reinterpret_cast<uintptr_t>(dev), r.end - r.begin);
+}
+
+// A kept plan between the header and the parameters of an FP64 user call that splits
+// nothing: 1 when any of the call's copies meets one of the plan's.
+void udf_next_to_plan() {
+  zmc_ctx *c = context(8 << 20, 13);
+  std::vector<zmc_desc> rows = gauss_rows(400, 1, 1);
+  for (size_t i = 0; i < 264; ++i) rows[i].n_samples = 2 * 2080 + 1;  // 928 chunks in all
+  zmc_plan *hole = plan(c, rows);
+  g_uploads.clear();
+  zmc_plan *kept = plan(c, gauss_rows(1, 1, 1));
+  const std::vector<Range> mine = g_uploads;
+  zmc_plan_destroy(hole);
+  g_uploads.clear();
+  std::vector<zmc_desc> user_rows = gauss_rows(440, 1, 1);
+  std::vector<UdfRow> ur(user_rows.size());
+  for (size_t i = 0; i < ur.size(); ++i) ur[i] = row_of(user_rows[i]);
+  std::vector<zmc_result> out(ur.size());
+  const zmc_status st = udf_run(c, user(ZMC_UDF_F64), ur.data(), ur.size(), out.data());
+  int met = 0;
+  for (const Range &a : g_uploads)
+    for (const Range &b : mine) met += a.meets(b);
+  std::printf("%d %d\n", st, met > 0);
+  zmc_plan_destroy(kept);
+  zmc_destroy(c);
+}
+
+}  // namespace
+
+int main(int, char **argv) {
+  const std::string what = argv[1];
+  if (what == "upload_gap") upload_gap();
+  if (what == "udf_next_to_plan") udf_next_to_plan();
+  return 0;
+}

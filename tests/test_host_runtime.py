@@ -1,0 +1,39 @@
+"""The host runtime's bookkeeping on the CPU: tests/helpers/host_runtime.cpp links the
+runtime against a CUDA whose device memory is host memory and whose copies and
+launches are only noted."""
+import os
+import subprocess
+
+import pytest
+
+from paper_2104_10073_gb300 import build
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+
+@pytest.fixture(scope="module")
+def run(tmp_path_factory):
+    build.build()  # writes the header with the run-time compiled sources
+    exe = str(tmp_path_factory.mktemp("host") / "host_runtime")
+    csrc = os.path.join(ROOT, "paper_2104_10073_gb300", "csrc")
+    subprocess.run(["g++", "-std=c++17", "-O1", "-pthread", "-I", os.path.join(ROOT, "include"),
+                    "-I", csrc, "-I", os.path.join(ROOT, "paper_2104_10073_gb300", "_build"),
+                    "-I", "/usr/local/cuda/include",
+                    os.path.join(ROOT, "tests", "helpers", "host_runtime.cpp"),
+                    *[os.path.join(csrc, f"zmc_{s}.cpp")
+                      for s in ("runtime", "tune", "pool", "polyroots")],
+                    "-o", exe, "-ldl"], check=True)
+
+    def call(*args):
+        out = subprocess.run([exe, *args], capture_output=True, text=True, check=True, timeout=60)
+        return out.stdout.splitlines()
+
+    return call
+
+
+def test_copies_join_only_what_is_consecutive(run):
+    assert run("upload_gap") == ["0 160", "2048 522"]
+
+
+def test_user_call_leaves_a_plan_between_its_tables_alone(run):
+    assert run("udf_next_to_plan") == ["0 0"]
