@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(256) zmc_finish_kernel(const Entry *__restrict
                      : "memory");
       before = __shfl_sync(kFullMask, before, 0);
       if (before != last) continue;
-      __threadfence();
+      __syncwarp();  // the shuffle orders no memory: all lanes after lane 0's acquire
       merge_row(en.fn, chunk_samples_of(Q), lane);
     } else {
       const uint32_t e = w - total;
