@@ -131,6 +131,7 @@ struct LaunchHdr {
   // part[f][32 (blocks per chunk t + b)].
   uint32_t split[4];
   float2 *part[4];
+  uint32_t *left;  // counts of the finish kernel, n_entries zeros, when any chunk is split
 };
 
 // FP64 descriptor of the plain per-integrand kernel (passed by value).
@@ -174,9 +175,9 @@ cudaError_t launch_batched(int family, const Entry *entries, LaunchHdr *hdr, uns
 cudaError_t launch_merge(const FnDev *const *fns, LaunchHdr *hdr, unsigned grid,
                          cudaStream_t stream, bool reset = false);
 // The records of a launch's split chunks and the merge of its rows (n_entries rows,
-// one entry each); warps: split chunks + rows; left: n_entries zeros.
-cudaError_t launch_finish(const Entry *entries, LaunchHdr *hdr, uint32_t *left, uint64_t warps,
-                          int sms, cudaStream_t stream);
+// one entry each); warps: split chunks + rows.
+cudaError_t launch_finish(const Entry *entries, LaunchHdr *hdr, uint64_t warps, int sms,
+                          cudaStream_t stream);
 cudaError_t launch_plain(const PlainFn &fn, double *block_rec, unsigned grid,
                          cudaStream_t stream);
 cudaError_t launch_plain_merge(const PlainJob *jobs, uint32_t n, cudaStream_t stream);

@@ -155,10 +155,9 @@ __global__ void __launch_bounds__(256) zmc_merge_kernel(const FnDev *const *__re
 // one warp per split chunk makes its record, and the warp that completes a row's
 // count of split chunks merges the row; one warp per row without any merges it at
 // once.  One kernel less than records and merge apart (~4 us of a small call).
-// left: a count per entry, zero before the first run; it wraps to zero by itself.
+// hdr->left: a count per entry, zero before the first run; it wraps to zero by itself.
 __global__ void __launch_bounds__(256) zmc_finish_kernel(const Entry *__restrict__ entries,
-                                                         LaunchHdr *__restrict__ hdr,
-                                                         uint32_t *__restrict__ left) {
+                                                         LaunchHdr *__restrict__ hdr) {
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
   const uint32_t Q = hdr->quints_per_lane;
@@ -186,7 +185,7 @@ __global__ void __launch_bounds__(256) zmc_finish_kernel(const Entry *__restrict
       if (lane == 0)  // after this lane's record
         asm volatile("atom.acq_rel.gpu.global.inc.u32 %0, [%1], %2;"
                      : "=r"(before)
-                     : "l"(left + e), "r"(last)
+                     : "l"(hdr->left + e), "r"(last)
                      : "memory");
       before = __shfl_sync(kFullMask, before, 0);
       if (before != last) continue;
@@ -265,10 +264,10 @@ cudaError_t launch_merge(const FnDev *const *fns, LaunchHdr *hdr, unsigned grid,
   return cudaGetLastError();
 }
 
-cudaError_t launch_finish(const Entry *entries, LaunchHdr *hdr, uint32_t *left, uint64_t warps,
-                          int sms, cudaStream_t stream) {
+cudaError_t launch_finish(const Entry *entries, LaunchHdr *hdr, uint64_t warps, int sms,
+                          cudaStream_t stream) {
   const uint64_t blocks = std::min<uint64_t>((warps + 7) / 8, 16ull * static_cast<unsigned>(sms));
-  zmc_finish_kernel<<<static_cast<unsigned>(blocks), 256, 0, stream>>>(entries, hdr, left);
+  zmc_finish_kernel<<<static_cast<unsigned>(blocks), 256, 0, stream>>>(entries, hdr);
   return cudaGetLastError();
 }
 

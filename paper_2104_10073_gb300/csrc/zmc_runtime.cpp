@@ -597,8 +597,8 @@ struct zmc_plan {
   uint64_t n_chunks = 0, n_samples = 0;
   uint64_t fam_items[4] = {0, 0, 0, 0};
   uint64_t fam_units[4] = {0, 0, 0, 0};  // whole chunks and blocks of split ones
-  void *d_part = nullptr;     // lane summaries of the split chunks
-  uint32_t *d_left = nullptr;  // counts of the finish kernel, when chunks may be split
+  bool splits = false;        // chunks may be split: the merge is the finish kernel
+  void *d_split = nullptr;    // their scratch (split_bytes)
   bool dirty = false;          // the counters were drawn from and not reset
   bool ranged = false;  // built by zmc_integrate_moments (no plain form)
   uint32_t quints = 0;  // chunk = 160 * quints samples
@@ -619,10 +619,10 @@ struct zmc_plan {
   void release_all() {
     for (void *p : blocks) ctx->arena.release(p);
     blocks.clear();
-    if (d_part) {
-      ctx->arena.release(d_part);
+    if (d_split) {
+      ctx->arena.release(d_split);
       ctx->split_plans.erase(this);
-      d_part = nullptr;
+      d_split = nullptr;
     }
   }
 };
@@ -637,8 +637,7 @@ static void drop_splits(zmc_ctx *ctx) {
     if (p->dirty) {  // sampled, not merged yet: the records are still to be made
       uint64_t warps = p->n;
       for (uint32_t k : p->h_hdr.split) warps += k;
-      ok = ok && launch_finish(p->d_entries, p->d_hdr, p->d_left, warps, ctx->sms, ctx->stream) ==
-                     cudaSuccess;
+      ok = ok && launch_finish(p->d_entries, p->d_hdr, warps, ctx->sms, ctx->stream) == cudaSuccess;
       p->dirty = false;
     }
     std::memset(p->h_hdr.split, 0, sizeof p->h_hdr.split);
@@ -648,8 +647,8 @@ static void drop_splits(zmc_ctx *ctx) {
   // launches already enqueued use the scratch
   if (cudaStreamSynchronize(ctx->stream) != cudaSuccess || !ok) return;
   for (zmc_plan *p : ctx->split_plans) {
-    ctx->arena.release(p->d_part);
-    p->d_part = nullptr;
+    ctx->arena.release(p->d_split);
+    p->d_split = nullptr;
   }
   ctx->split_plans.clear();
 }
@@ -1069,14 +1068,7 @@ zmc_status plan_build(zmc_ctx *ctx, const zmc_desc *desc, size_t n, zmc_plan **o
                             static_cast<uint64_t>(ctx->sms) * 8 * std::max(bps, 1), plan->quints);
     n_split += split[f];
   }
-  // the header and, after it, the finish kernel's counts; no room for those: no split
-  size_t hdr_bytes = sizeof(LaunchHdr) + (n_split ? n * sizeof(uint32_t) : 0);
-  plan->d_hdr = static_cast<LaunchHdr *>(plan->alloc(hdr_bytes));
-  if (!plan->d_hdr && n_split) {
-    n_split = 0;
-    hdr_bytes = sizeof(LaunchHdr);
-    plan->d_hdr = static_cast<LaunchHdr *>(plan->alloc(hdr_bytes));
-  }
+  plan->d_hdr = static_cast<LaunchHdr *>(plan->alloc(sizeof(LaunchHdr)));
   if (!plan->d_fns || !plan->d_rec || (keep && !plan->d_out) || !plan->d_entries ||
       !plan->d_merge || !plan->d_hdr) {
     plan->release_all();
@@ -1084,11 +1076,13 @@ zmc_status plan_build(zmc_ctx *ctx, const zmc_desc *desc, size_t n, zmc_plan **o
                      (fn_bytes + total * 8.0 + n * 64.0) / 1e6,
                      ctx->arena.largest_free() / 1e6);
   }
-  // pinned staging: the tables at the arena's granularity, then the results of a
-  // plan that goes before the call returns, which the merge writes straight to the
-  // host (no copy back)
+  // pinned staging: the tables at the arena's granularity, the zeros of the finish
+  // kernel's counts, then the results of a plan that goes before the call returns,
+  // which the merge writes straight to the host (no copy back)
+  const size_t left_bytes = n_split ? n * sizeof(uint32_t) : 0;
   const size_t o_ent = round256(fn_bytes), o_mrg = o_ent + round256(ent_bytes),
-               o_hdr = o_mrg + round256(mrg_bytes), o_res = o_hdr + round256(hdr_bytes);
+               o_hdr = o_mrg + round256(mrg_bytes), o_left = o_hdr + round256(sizeof(LaunchHdr)),
+               o_res = o_left + round256(left_bytes);
   zmc_status st = ensure_stage(ctx, o_res + (keep ? 0 : n * sizeof(zmc_result)));
   if (st != ZMC_OK) {
     plan->release_all();
@@ -1150,17 +1144,18 @@ zmc_status plan_build(zmc_ctx *ctx, const zmc_desc *desc, size_t n, zmc_plan **o
   // room for it every chunk stays whole (arena_take takes it back when a later
   // table needs the room; the serving scheduler cannot, so a plan of a serving
   // context that outlives the call has none)
-  const size_t nb = chunk_blocks(plan->quints);
   if (n_split && !(ctx->serving && keep))
-    plan->d_part = ctx->arena.alloc(n_split * nb * kPartBytes);
-  if (plan->d_part) {
+    plan->d_split = ctx->arena.alloc(split_bytes(n, n_split, plan->quints));
+  if (plan->d_split) {
+    plan->splits = true;
     ctx->split_plans.insert(plan.get());
-    plan->d_left = reinterpret_cast<uint32_t *>(plan->d_hdr + 1);
-    auto *part = static_cast<float2 *>(plan->d_part);
+    h.left = static_cast<uint32_t *>(plan->d_split);
+    auto *part = reinterpret_cast<float2 *>(static_cast<char *>(plan->d_split) +
+                                            round256(n * sizeof(uint32_t)));
     for (int f = 0; f < 4; ++f) {
       h.split[f] = split[f];
       h.part[f] = part;
-      part += split[f] * nb * 32;
+      part += static_cast<size_t>(split[f]) * chunk_blocks(plan->quints) * 32;
     }
   }
   for (int f = 0; f < 4; ++f) {
@@ -1189,13 +1184,14 @@ zmc_status plan_build(zmc_ctx *ctx, const zmc_desc *desc, size_t n, zmc_plan **o
   std::memcpy(s + o_ent, ents.data(), ent_bytes);
   std::memcpy(s + o_mrg, merge.data(), mrg_bytes);
   std::memcpy(s + o_hdr, &h, sizeof h);
-  std::memset(s + o_hdr + sizeof h, 0, hdr_bytes - sizeof h);
+  std::memset(s + o_left, 0, left_bytes);
   cudaStream_t str = ctx->stream;
   const UploadPart parts[] = {{plan->d_fns, 0, fn_bytes},
                               {plan->d_entries, o_ent, ent_bytes},
                               {plan->d_merge, o_mrg, mrg_bytes},
-                              {plan->d_hdr, o_hdr, hdr_bytes}};
-  cudaError_t e = upload_parts(parts, 4, s, str);
+                              {plan->d_hdr, o_hdr, sizeof h},
+                              {plan->d_split, o_left, left_bytes}};
+  cudaError_t e = upload_parts(parts, plan->d_split ? 5 : 4, s, str);
   // keep = false: nothing writes the staging's tables before the caller has waited
   if (e == cudaSuccess && keep) e = cudaStreamSynchronize(str);
   if (e != cudaSuccess) {
@@ -1236,10 +1232,10 @@ zmc_status plan_enqueue(zmc_plan *plan, uint32_t stages) {
                                   plan->block, present, str, plan->unroll));
   }
   if (stages & ZMC_STAGE_MERGE) {
-    if (plan->d_left) {  // also after the scratch went: then every row merges at once
+    if (plan->splits) {  // also after the scratch went: then every row merges at once
       uint64_t warps = plan->n;
       for (uint32_t k : plan->h_hdr.split) warps += k;
-      ZMC_CUDA(ctx, launch_finish(plan->d_entries, plan->d_hdr, plan->d_left, warps, ctx->sms, str));
+      ZMC_CUDA(ctx, launch_finish(plan->d_entries, plan->d_hdr, warps, ctx->sms, str));
     } else {
       const unsigned grid = static_cast<unsigned>(
           std::min<size_t>((plan->n + 7) / 8, static_cast<size_t>(ctx->sms) * 16));

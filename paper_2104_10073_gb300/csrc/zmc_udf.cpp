@@ -245,7 +245,6 @@ zmc_status udf_run(zmc_ctx *ctx, const zmc_udf *udf, const UdfRow *rows, size_t 
 
   const bool f64 = udf->precision == ZMC_UDF_F64;
   const uint64_t chunk = chunk_samples_of(ctx->quints_per_lane);
-  size_t hdr_b = sizeof(LaunchHdr) + n * sizeof(uint32_t);  // + the finish kernel's counts
   std::vector<uint32_t> prow(f64 ? n : 0);  // FP64: index of the row's parameter block
   std::vector<const double *> params;       // distinct parameter arrays, in first-use order
   for (size_t i = 0; f64 && i < n; ++i) {
@@ -257,11 +256,11 @@ zmc_status udf_run(zmc_ctx *ctx, const zmc_udf *udf, const UdfRow *rows, size_t 
   }
   const size_t fn_b = n * sizeof(FnDev), ent_b = n * sizeof(Entry), mrg_b = n * sizeof(FnDev *),
                p_b = params.size() * ZMC_NPARAM * sizeof(double);
-  // host tables in the pinned staging buffer: fns | entries | merge list | hdr | params,
-  // then the results, which the merge writes there
+  // host tables in the pinned staging buffer: fns | entries | merge list | hdr | params |
+  // zeros of the finish kernel's counts, then the results, which the merge writes there
   const size_t o_ent = round256(fn_b), o_mrg = o_ent + round256(ent_b),
-               o_hdr = o_mrg + round256(mrg_b), o_p = o_hdr + round256(hdr_b),
-               o_res = o_p + round256(p_b);
+               o_hdr = o_mrg + round256(mrg_b), o_p = o_hdr + round256(sizeof(LaunchHdr)),
+               o_left = o_p + round256(p_b), o_res = o_left + round256(n * sizeof(uint32_t));
   st = ensure_stage(ctx, o_res + n * sizeof(zmc_result));
   if (st != ZMC_OK) return st;
   char *s = static_cast<char *>(ctx->stage);
@@ -299,13 +298,7 @@ zmc_status udf_run(zmc_ctx *ctx, const zmc_udf *udf, const UdfRow *rows, size_t 
   auto *d_mrg = static_cast<const FnDev **>(ab.get(mrg_b));
   const uint64_t resident = static_cast<uint64_t>(ctx->sms) * udf->max_blocks * 8;
   uint32_t split = split_chunks(total, alike, resident, ctx->quints_per_lane);
-  if (!split) hdr_b = sizeof(LaunchHdr);
-  auto *d_hdr = static_cast<LaunchHdr *>(ab.get(hdr_b));
-  if (!d_hdr && split) {  // no room for the counts: no split
-    split = 0;
-    hdr_b = sizeof(LaunchHdr);
-    d_hdr = static_cast<LaunchHdr *>(ab.get(hdr_b));
-  }
+  auto *d_hdr = static_cast<LaunchHdr *>(ab.get(sizeof(LaunchHdr)));
   auto *d_p = static_cast<double *>(p_b ? ab.get(p_b) : nullptr);
   if (!d_fns || !d_rec || !d_ent || !d_mrg || !d_hdr || (p_b && !d_p))
     return set_error(ZMC_ENOMEM, "udf call needs %.1f MB of device memory",
@@ -337,31 +330,35 @@ zmc_status udf_run(zmc_ctx *ctx, const zmc_udf *udf, const UdfRow *rows, size_t 
     ents[k].chunk_begin = 0;
     item += (rows[i].n_samples + chunk - 1) / chunk;
   }
-  std::memset(hdr, 0, hdr_b);
+  std::memset(hdr, 0, sizeof *hdr);
   // without room for their scratch, all chunks stay whole
-  float2 *d_part = nullptr;
+  const size_t left_b = round256(n * sizeof(uint32_t));
+  char *d_split = nullptr;
   if (split) {
-    d_part = static_cast<float2 *>(
-        ctx->arena.alloc(split * chunk_blocks(ctx->quints_per_lane) * kPartBytes));
-    if (d_part)
-      ab.held.push_back(d_part);
-    else
+    d_split = static_cast<char *>(ctx->arena.alloc(split_bytes(n, split, ctx->quints_per_lane)));
+    if (d_split) {
+      ab.held.push_back(d_split);
+      std::memset(s + o_left, 0, left_b);
+      hdr->split[0] = split;
+      hdr->part[0] = reinterpret_cast<float2 *>(d_split + left_b);
+      hdr->left = reinterpret_cast<uint32_t *>(d_split);
+    } else {
       split = 0;
+    }
   }
-  hdr->split[0] = split;
-  hdr->part[0] = d_part;
   hdr->item_end[0] = item;
   hdr->n_entries = static_cast<uint32_t>(n);
   hdr->n_merge = static_cast<uint32_t>(n);
   hdr->quints_per_lane = ctx->quints_per_lane;
 
   cudaStream_t str = ctx->stream;
-  const UploadPart parts[] = {{d_fns, 0, fn_b},
-                              {d_ent, o_ent, ent_b},
-                              {d_mrg, o_mrg, mrg_b},
-                              {d_hdr, o_hdr, hdr_b},
-                              {d_p, o_p, p_b}};
-  e = upload_parts(parts, p_b ? 5 : 4, s, str);
+  std::vector<UploadPart> parts = {{d_fns, 0, fn_b},
+                                   {d_ent, o_ent, ent_b},
+                                   {d_mrg, o_mrg, mrg_b},
+                                   {d_hdr, o_hdr, sizeof *hdr}};
+  if (p_b) parts.push_back({d_p, o_p, p_b});
+  if (split) parts.push_back({d_split, o_left, left_b});
+  e = upload_parts(parts.data(), parts.size(), s, str);
   if (e == cudaSuccess) {
     // persistent grid: the kernel's occupancy, no more warps than work items
     const uint64_t units = launch_units(item, split, ctx->quints_per_lane);
@@ -376,8 +373,7 @@ zmc_status udf_run(zmc_ctx *ctx, const zmc_udf *udf, const UdfRow *rows, size_t 
                          args, 0, str);
   }
   if (e == cudaSuccess && split) {
-    e = launch_finish(d_ent, d_hdr, reinterpret_cast<uint32_t *>(d_hdr + 1), n + split, ctx->sms,
-                      str);
+    e = launch_finish(d_ent, d_hdr, n + split, ctx->sms, str);
   } else if (e == cudaSuccess) {
     const unsigned mg = static_cast<unsigned>(
         std::min<uint64_t>((n + 7) / 8, static_cast<uint64_t>(ctx->sms) * 16));

@@ -108,7 +108,7 @@ cudaError_t launch_merge(const FnDev *const *, LaunchHdr *h, unsigned, cudaStrea
   if (reset) std::memset(h->counter, 0, sizeof h->counter);
   return cudaSuccess;
 }
-cudaError_t launch_finish(const Entry *, LaunchHdr *h, uint32_t *, uint64_t, int, cudaStream_t) {
+cudaError_t launch_finish(const Entry *, LaunchHdr *h, uint64_t, int, cudaStream_t) {
   note("finish split %u", splits(h));
   std::memset(h->counter, 0, sizeof h->counter);
   return cudaSuccess;
@@ -205,11 +205,39 @@ void udf_next_to_plan() {
   zmc_destroy(c);
 }
 
+// Two tables that exactly fill the arena, the first with chunks to split: 1 when the
+// second is taken as well.
+std::vector<zmc_desc> unlike_rows(size_t n) {
+  std::vector<zmc_desc> rows = gauss_rows(n, 1, 1);
+  for (size_t i = 0; i < n; i += 2) rows[i] = gauss_rows(1, 7, 1)[0];
+  return rows;
+}
+size_t table_bytes(size_t n) {  // records, results, descriptors, entries, merge list, header
+  return round256(n * 8) + round256(n * sizeof(zmc_result)) + round256(n * sizeof(FnDev)) +
+         round256(n * sizeof(Entry)) + round256(n * 8) + 256;
+}
+void two_tables(bool serving) {
+  zmc_options o;
+  zmc_default_options(&o);
+  o.mem_budget_bytes = 2 * table_bytes(1000);
+  o.quints_per_lane = 104;
+  o.serving = serving;
+  zmc_ctx *c = nullptr;
+  if (zmc_create(&o, &c) != ZMC_OK) std::abort();
+  zmc_plan *a = plan(c, unlike_rows(1000)), *b = plan(c, unlike_rows(1000));
+  std::printf("%d %d\n", a != nullptr, b != nullptr);
+  zmc_plan_destroy(a);
+  zmc_plan_destroy(b);
+  zmc_destroy(c);
+}
+
 }  // namespace
 
 int main(int, char **argv) {
   const std::string what = argv[1];
   if (what == "upload_gap") upload_gap();
   if (what == "udf_next_to_plan") udf_next_to_plan();
+  if (what == "two_tables") two_tables(false);
+  if (what == "two_serving_tables") two_tables(true);
   return 0;
 }

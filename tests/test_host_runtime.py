@@ -37,3 +37,8 @@ def test_copies_join_only_what_is_consecutive(run):
 
 def test_user_call_leaves_a_plan_between_its_tables_alone(run):
     assert run("udf_next_to_plan") == ["0 0"]
+
+
+@pytest.mark.parametrize("context", ["two_tables", "two_serving_tables"])
+def test_a_plans_scratch_takes_no_room_from_a_later_table(run, context):
+    assert run(context) == ["1 1"]
