@@ -175,9 +175,9 @@ cudaError_t launch_batched(int family, const Entry *entries, LaunchHdr *hdr, uns
 cudaError_t launch_merge(const FnDev *const *fns, LaunchHdr *hdr, unsigned grid,
                          cudaStream_t stream, bool reset = false);
 // The records of a launch's split chunks and the merge of its rows (n_entries rows,
-// one entry each); warps: split chunks + rows.
+// one entry each); warps: split chunks + rows.  merge = false: the records alone.
 cudaError_t launch_finish(const Entry *entries, LaunchHdr *hdr, uint64_t warps, int sms,
-                          cudaStream_t stream);
+                          cudaStream_t stream, bool merge = true);
 cudaError_t launch_plain(const PlainFn &fn, double *block_rec, unsigned grid,
                          cudaStream_t stream);
 cudaError_t launch_plain_merge(const PlainJob *jobs, uint32_t n, cudaStream_t stream);

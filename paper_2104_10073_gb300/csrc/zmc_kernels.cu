@@ -156,8 +156,9 @@ __global__ void __launch_bounds__(256) zmc_merge_kernel(const FnDev *const *__re
 // count of split chunks merges the row; one warp per row without any merges it at
 // once.  One kernel less than records and merge apart (~4 us of a small call).
 // hdr->left: a count per entry, zero before the first run; it wraps to zero by itself.
+// merge = false: the records alone, no result is written.
 __global__ void __launch_bounds__(256) zmc_finish_kernel(const Entry *__restrict__ entries,
-                                                         LaunchHdr *__restrict__ hdr) {
+                                                         LaunchHdr *__restrict__ hdr, bool merge) {
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t nwarps = (gridDim.x * blockDim.x) >> 5;
   const uint32_t Q = hdr->quints_per_lane;
@@ -166,7 +167,7 @@ __global__ void __launch_bounds__(256) zmc_finish_kernel(const Entry *__restrict
   for (int f = 0; f < 4; ++f) total += hdr->split[f];
   uint32_t w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   if (w == 0 && lane < 4) hdr->counter[lane] = 0;
-  for (; w < total + ne; w += nwarps) {
+  for (; w < total + (merge ? ne : 0u); w += nwarps) {
     if (w < total) {
       int f = 0;
       uint32_t t = w;
@@ -177,6 +178,7 @@ __global__ void __launch_bounds__(256) zmc_finish_kernel(const Entry *__restrict
       const uint64_t chunk = en.chunk_begin + (split0 + t - en.item_begin);
       combine_blocks(en.fn, chunk, samples_of(en.fn, chunk, Q), Q, lane,
                      hdr->part[f] + static_cast<size_t>(t) * 32u * chunk_blocks(Q));
+      if (!merge) continue;
       const uint64_t next = e + 1 < ne ? entries[e + 1].item_begin : hdr->item_end[f];
       const uint64_t end = next < hdr->item_end[f] ? next : hdr->item_end[f];
       const uint32_t last =
@@ -265,9 +267,9 @@ cudaError_t launch_merge(const FnDev *const *fns, LaunchHdr *hdr, unsigned grid,
 }
 
 cudaError_t launch_finish(const Entry *entries, LaunchHdr *hdr, uint64_t warps, int sms,
-                          cudaStream_t stream) {
+                          cudaStream_t stream, bool merge) {
   const uint64_t blocks = std::min<uint64_t>((warps + 7) / 8, 16ull * static_cast<unsigned>(sms));
-  zmc_finish_kernel<<<static_cast<unsigned>(blocks), 256, 0, stream>>>(entries, hdr);
+  zmc_finish_kernel<<<static_cast<unsigned>(blocks), 256, 0, stream>>>(entries, hdr, merge);
   return cudaGetLastError();
 }
 

@@ -634,10 +634,12 @@ namespace zmc {
 static void drop_splits(zmc_ctx *ctx) {
   bool ok = true;
   for (zmc_plan *p : ctx->split_plans) {
-    if (p->dirty) {  // sampled, not merged yet: the records are still to be made
+    if (p->dirty) {  // sampled, not merged yet: the records are still to be made (a merge
+                     // that nobody asked for would write over the plan's results)
       uint64_t warps = p->n;
       for (uint32_t k : p->h_hdr.split) warps += k;
-      ok = ok && launch_finish(p->d_entries, p->d_hdr, warps, ctx->sms, ctx->stream) == cudaSuccess;
+      ok = ok && launch_finish(p->d_entries, p->d_hdr, warps, ctx->sms, ctx->stream, false) ==
+                     cudaSuccess;
       p->dirty = false;
     }
     std::memset(p->h_hdr.split, 0, sizeof p->h_hdr.split);

@@ -108,8 +108,8 @@ cudaError_t launch_merge(const FnDev *const *, LaunchHdr *h, unsigned, cudaStrea
   if (reset) std::memset(h->counter, 0, sizeof h->counter);
   return cudaSuccess;
 }
-cudaError_t launch_finish(const Entry *, LaunchHdr *h, uint64_t, int, cudaStream_t) {
-  note("finish split %u", splits(h));
+cudaError_t launch_finish(const Entry *, LaunchHdr *h, uint64_t, int, cudaStream_t, bool merge) {
+  note("%s split %u", merge ? "finish" : "records", splits(h));
   std::memset(h->counter, 0, sizeof h->counter);
   return cudaSuccess;
 }
@@ -231,6 +231,20 @@ void two_tables(bool serving) {
   zmc_destroy(c);
 }
 
+// A sampled plan whose scratch a later table takes: what was launched for it.
+void scratch_taken_after_sampling() {
+  zmc_ctx *c = context(table_bytes(1000) + split_bytes(1000, 1000, 104) + 4096, 104);
+  zmc_plan *a = plan(c, unlike_rows(1000));
+  zmc_plan_run(a, ZMC_STAGE_SAMPLE);
+  g_events.clear();
+  zmc_plan *b = plan(c, unlike_rows(1000));
+  std::printf("%d\n", b != nullptr);
+  for (const std::string &e : g_events) std::printf("%s\n", e.c_str());
+  zmc_plan_destroy(a);
+  zmc_plan_destroy(b);
+  zmc_destroy(c);
+}
+
 }  // namespace
 
 int main(int, char **argv) {
@@ -239,5 +253,6 @@ int main(int, char **argv) {
   if (what == "udf_next_to_plan") udf_next_to_plan();
   if (what == "two_tables") two_tables(false);
   if (what == "two_serving_tables") two_tables(true);
+  if (what == "scratch_taken_after_sampling") scratch_taken_after_sampling();
   return 0;
 }

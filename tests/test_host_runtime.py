@@ -42,3 +42,7 @@ def test_user_call_leaves_a_plan_between_its_tables_alone(run):
 @pytest.mark.parametrize("context", ["two_tables", "two_serving_tables"])
 def test_a_plans_scratch_takes_no_room_from_a_later_table(run, context):
     assert run(context) == ["1 1"]
+
+
+def test_taking_scratch_back_makes_records_and_writes_no_result(run):
+    assert run("scratch_taken_after_sampling") == ["1", "records split 1000"]
