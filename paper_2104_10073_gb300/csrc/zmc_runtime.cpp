@@ -92,6 +92,22 @@ void Arena::release(void *p) {
   free_[start] = len;
 }
 
+bool Arena::fits_without(const std::vector<void *> &blocks, size_t bytes) const {
+  std::lock_guard<std::mutex> g(mu_);
+  std::map<size_t, size_t> ranges = free_;
+  for (const void *p : blocks) {
+    const auto a = allocated_.find(static_cast<size_t>(static_cast<const char *>(p) - base_));
+    if (a != allocated_.end()) ranges.insert(*a);
+  }
+  size_t end = 0, run = 0;  // the run of free bytes that ends here
+  for (const auto &r : ranges) {
+    run = r.first == end ? run + r.second : r.second;
+    end = r.first + r.second;
+    if (run >= bytes) return true;
+  }
+  return false;
+}
+
 size_t Arena::largest_free() const {
   std::lock_guard<std::mutex> g(mu_);
   size_t m = 0;
@@ -598,7 +614,8 @@ struct zmc_plan {
   uint64_t fam_items[4] = {0, 0, 0, 0};
   uint64_t fam_units[4] = {0, 0, 0, 0};  // whole chunks and blocks of split ones
   bool splits = false;        // chunks may be split: the merge is the finish kernel
-  void *d_split = nullptr;    // their scratch (split_bytes)
+  void *d_split = nullptr;    // their scratch
+  size_t scratch_bytes = 0;   // its size (split_bytes)
   bool dirty = false;          // the counters were drawn from and not reset
   bool ranged = false;  // built by zmc_integrate_moments (no plain form)
   uint32_t quints = 0;  // chunk = 160 * quints samples
@@ -629,11 +646,22 @@ struct zmc_plan {
 
 namespace zmc {
 
-// Gives the scratch of every plan back to the arena: from the next run on, those
-// plans hand out whole chunks only.
-static void drop_splits(zmc_ctx *ctx) {
+// Gives plans' scratch back to the arena, of as few plans as make room for `bytes`, of
+// none when all of it would not: from the next run on, those plans hand out whole
+// chunks only.
+static void drop_splits(zmc_ctx *ctx, size_t bytes) {
+  std::vector<zmc_plan *> drop(ctx->split_plans.begin(), ctx->split_plans.end());
+  const auto fits = [&](const zmc_plan *but) {
+    std::vector<void *> blocks;
+    for (const zmc_plan *p : drop)
+      if (p != but) blocks.push_back(p->d_split);
+    return ctx->arena.fits_without(blocks, bytes);
+  };
+  if (!fits(nullptr)) return;
+  for (size_t k = drop.size(); k-- > 0;)
+    if (fits(drop[k])) drop.erase(drop.begin() + static_cast<ptrdiff_t>(k));
   bool ok = true;
-  for (zmc_plan *p : ctx->split_plans) {
+  for (zmc_plan *p : drop) {
     if (p->dirty) {  // sampled, not merged yet: the records are still to be made (a merge
                      // that nobody asked for would write over the plan's results)
       uint64_t warps = p->n;
@@ -648,20 +676,26 @@ static void drop_splits(zmc_ctx *ctx) {
   }
   // launches already enqueued use the scratch
   if (cudaStreamSynchronize(ctx->stream) != cudaSuccess || !ok) return;
-  for (zmc_plan *p : ctx->split_plans) {
+  for (zmc_plan *p : drop) {
     ctx->arena.release(p->d_split);
     p->d_split = nullptr;
+    ctx->split_plans.erase(p);
   }
-  ctx->split_plans.clear();
 }
 
 void *arena_take(zmc_ctx *ctx, size_t bytes) {
   void *p = ctx->arena.alloc(bytes);
   if (!p && !ctx->split_plans.empty()) {
-    drop_splits(ctx);
+    drop_splits(ctx, bytes);
     p = ctx->arena.alloc(bytes);
   }
   return p;
+}
+
+bool arena_could_hold(const zmc_ctx *ctx, size_t bytes) {
+  size_t room = ctx->arena.size() - ctx->arena.used();
+  for (const zmc_plan *p : ctx->split_plans) room += round256(p->scratch_bytes);
+  return bytes <= room;
 }
 
 }  // namespace zmc
@@ -1046,6 +1080,17 @@ zmc_status plan_build(zmc_ctx *ctx, const zmc_desc *desc, size_t n, zmc_plan **o
   const size_t fn_bytes = n * sizeof(FnDev);
   const size_t ent_bytes = n * sizeof(Entry);
   const size_t mrg_bytes = n * sizeof(FnDev *);
+  const auto no_room = [&] {
+    plan->release_all();
+    return set_error(ZMC_ENOMEM, "plan needs %.1f MB of device memory; arena has %.1f MB free",
+                     (fn_bytes + total * 8.0 + n * 64.0) / 1e6,
+                     ctx->arena.largest_free() / 1e6);
+  };
+  if (!arena_could_hold(ctx, round256(total * sizeof(float2)) + round256(fn_bytes) +
+                                 round256(ent_bytes) + round256(mrg_bytes) +
+                                 round256(sizeof(LaunchHdr)) +
+                                 (keep ? round256(n * sizeof(zmc_result)) : 0)))
+    return no_room();
   plan->d_rec = static_cast<float2 *>(plan->alloc(total * sizeof(float2)));
   if (keep) plan->d_out = static_cast<zmc_result *>(plan->alloc(n * sizeof(zmc_result)));
   // the uploaded tables one after the other, so that they are usually adjacent
@@ -1072,12 +1117,8 @@ zmc_status plan_build(zmc_ctx *ctx, const zmc_desc *desc, size_t n, zmc_plan **o
   }
   plan->d_hdr = static_cast<LaunchHdr *>(plan->alloc(sizeof(LaunchHdr)));
   if (!plan->d_fns || !plan->d_rec || (keep && !plan->d_out) || !plan->d_entries ||
-      !plan->d_merge || !plan->d_hdr) {
-    plan->release_all();
-    return set_error(ZMC_ENOMEM, "plan needs %.1f MB of device memory; arena has %.1f MB free",
-                     (fn_bytes + total * 8.0 + n * 64.0) / 1e6,
-                     ctx->arena.largest_free() / 1e6);
-  }
+      !plan->d_merge || !plan->d_hdr)
+    return no_room();
   // pinned staging: the tables at the arena's granularity, the zeros of the finish
   // kernel's counts, then the results of a plan that goes before the call returns,
   // which the merge writes straight to the host (no copy back)
@@ -1149,6 +1190,7 @@ zmc_status plan_build(zmc_ctx *ctx, const zmc_desc *desc, size_t n, zmc_plan **o
   if (n_split && !(ctx->serving && keep))
     plan->d_split = ctx->arena.alloc(split_bytes(n, n_split, plan->quints));
   if (plan->d_split) {
+    plan->scratch_bytes = split_bytes(n, n_split, plan->quints);
     plan->splits = true;
     ctx->split_plans.insert(plan.get());
     h.left = static_cast<uint32_t *>(plan->d_split);

@@ -30,6 +30,8 @@ class Arena {
   // nullptr when no free range is large enough.
   void *alloc(size_t bytes);
   void release(void *p);
+  // Whether alloc(bytes) would succeed if these blocks were free.
+  bool fits_without(const std::vector<void *> &blocks, size_t bytes) const;
   size_t used() const { return used_; }
   size_t size() const { return size_; }
   size_t largest_free() const;
@@ -147,6 +149,9 @@ cudaError_t upload_parts(const UploadPart *parts, size_t n, const char *stage, c
 // Device memory for a table from the context's arena, taking back the plans' split
 // scratch when there is no room otherwise (under api_mu).
 void *arena_take(zmc_ctx *ctx, size_t bytes);
+// Whether blocks of `bytes` in all could be taken so.  Asked before a table's first
+// block: a table that cannot fit takes no plan's scratch.
+bool arena_could_hold(const zmc_ctx *ctx, size_t bytes);
 // Chunks that are handed out by accumulation blocks (LaunchHdr::split).
 constexpr size_t kPartBytes = 32 * sizeof(float2);  // the lane summaries of one block
 constexpr uint64_t kSplitBytes = 8u << 20;          // at most, per family

@@ -290,6 +290,13 @@ zmc_status udf_run(zmc_ctx *ctx, const zmc_udf *udf, const UdfRow *rows, size_t 
     alike = alike && fns[i].variant == fns[0].variant;
     sorted = sorted && (i == 0 || fns[i - 1].variant <= fns[i].variant);
   }
+  const auto no_room = [&] {
+    return set_error(ZMC_ENOMEM, "udf call needs %.1f MB of device memory",
+                     (fn_b + total * 8.0 + n * 64.0 + p_b) / 1e6);
+  };
+  if (!arena_could_hold(ctx, round256(total * sizeof(float2)) + round256(fn_b) + round256(ent_b) +
+                                 round256(mrg_b) + round256(sizeof(LaunchHdr)) + round256(p_b)))
+    return no_room();
   ArenaBlocks ab{ctx, {}};
   auto *d_rec = static_cast<float2 *>(ab.get(total * sizeof(float2)));
   // the uploaded tables one after the other, so that they are usually adjacent
@@ -301,8 +308,7 @@ zmc_status udf_run(zmc_ctx *ctx, const zmc_udf *udf, const UdfRow *rows, size_t 
   auto *d_hdr = static_cast<LaunchHdr *>(ab.get(sizeof(LaunchHdr)));
   auto *d_p = static_cast<double *>(p_b ? ab.get(p_b) : nullptr);
   if (!d_fns || !d_rec || !d_ent || !d_mrg || !d_hdr || (p_b && !d_p))
-    return set_error(ZMC_ENOMEM, "udf call needs %.1f MB of device memory",
-                     (fn_b + total * 8.0 + n * 64.0 + p_b) / 1e6);
+    return no_room();
   for (size_t q = 0; q < params.size(); ++q)
     std::memcpy(ps + q * ZMC_NPARAM, params[q], ZMC_NPARAM * sizeof(double));
   uint64_t rec = 0;

@@ -245,6 +245,33 @@ void scratch_taken_after_sampling() {
   zmc_destroy(c);
 }
 
+// Split chunks that a plan's next sampling hands out.
+unsigned split_of(zmc_plan *p) {
+  g_events.clear();
+  zmc_plan_run(p, ZMC_STAGE_SAMPLE);
+  unsigned n = 0, f = 0, k = 0;
+  for (const std::string &e : g_events)
+    if (std::sscanf(e.c_str(), "batched %u split %u", &f, &k) == 2) n += k;
+  return n;
+}
+
+// Three plans with scratch, and a table that has room after one of them gave its back
+// (rows) or that has no room whatever they give.
+void scratch_taken_from(size_t rows) {
+  const size_t one = table_bytes(1000) + split_bytes(1000, 1000, 104);
+  zmc_ctx *c = context(3 * one + 4096, 104);
+  zmc_plan *a[3], *b;
+  for (zmc_plan *&p : a) p = plan(c, unlike_rows(1000));
+  b = plan(c, unlike_rows(rows));
+  std::printf("%d\n", b != nullptr);
+  unsigned whole = 0;
+  for (zmc_plan *p : a) whole += split_of(p) == 0;
+  std::printf("%u\n", whole);
+  for (zmc_plan *p : a) zmc_plan_destroy(p);
+  zmc_plan_destroy(b);
+  zmc_destroy(c);
+}
+
 }  // namespace
 
 int main(int, char **argv) {
@@ -254,5 +281,6 @@ int main(int, char **argv) {
   if (what == "two_tables") two_tables(false);
   if (what == "two_serving_tables") two_tables(true);
   if (what == "scratch_taken_after_sampling") scratch_taken_after_sampling();
+  if (what == "scratch_taken_from") scratch_taken_from(std::strtoul(argv[2], nullptr, 10));
   return 0;
 }

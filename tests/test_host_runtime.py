@@ -46,3 +46,8 @@ def test_a_plans_scratch_takes_no_room_from_a_later_table(run, context):
 
 def test_taking_scratch_back_makes_records_and_writes_no_result(run):
     assert run("scratch_taken_after_sampling") == ["1", "records split 1000"]
+
+
+@pytest.mark.parametrize("rows,taken,whole", [(1000, 1, 1), (100000, 0, 0)])
+def test_no_more_scratch_is_taken_back_than_makes_room(run, rows, taken, whole):
+    assert run("scratch_taken_from", str(rows)) == [str(taken), str(whole)]
