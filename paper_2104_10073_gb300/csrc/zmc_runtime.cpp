@@ -660,22 +660,27 @@ static void drop_splits(zmc_ctx *ctx, size_t bytes) {
   if (!fits(nullptr)) return;
   for (size_t k = drop.size(); k-- > 0;)
     if (fits(drop[k])) drop.erase(drop.begin() + static_cast<ptrdiff_t>(k));
-  bool ok = true;
+  cudaError_t e = cudaSuccess;
   for (zmc_plan *p : drop) {
-    if (p->dirty) {  // sampled, not merged yet: the records are still to be made (a merge
-                     // that nobody asked for would write over the plan's results)
+    if (e == cudaSuccess && p->dirty) {
+      // sampled, not merged yet: the records are still to be made (a merge that nobody
+      // asked for would write over the plan's results)
       uint64_t warps = p->n;
       for (uint32_t k : p->h_hdr.split) warps += k;
-      ok = ok && launch_finish(p->d_entries, p->d_hdr, warps, ctx->sms, ctx->stream, false) ==
-                     cudaSuccess;
+      e = launch_finish(p->d_entries, p->d_hdr, warps, ctx->sms, ctx->stream, false);
       p->dirty = false;
     }
     std::memset(p->h_hdr.split, 0, sizeof p->h_hdr.split);
-    ok = ok && cudaMemcpyAsync(p->d_hdr, &p->h_hdr, sizeof p->h_hdr, cudaMemcpyHostToDevice,
-                               ctx->stream) == cudaSuccess;
+    if (e == cudaSuccess)
+      e = cudaMemcpyAsync(p->d_hdr, &p->h_hdr, sizeof p->h_hdr, cudaMemcpyHostToDevice,
+                          ctx->stream);
   }
   // launches already enqueued use the scratch
-  if (cudaStreamSynchronize(ctx->stream) != cudaSuccess || !ok) return;
+  if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
+  if (e != cudaSuccess) {
+    ctx_cuda_fail(ctx, e, "taking back split scratch");
+    return;
+  }
   for (zmc_plan *p : drop) {
     ctx->arena.release(p->d_split);
     p->d_split = nullptr;
@@ -1082,6 +1087,7 @@ zmc_status plan_build(zmc_ctx *ctx, const zmc_desc *desc, size_t n, zmc_plan **o
   const size_t mrg_bytes = n * sizeof(FnDev *);
   const auto no_room = [&] {
     plan->release_all();
+    if (ctx->poisoned) return ZMC_ECUDA;
     return set_error(ZMC_ENOMEM, "plan needs %.1f MB of device memory; arena has %.1f MB free",
                      (fn_bytes + total * 8.0 + n * 64.0) / 1e6,
                      ctx->arena.largest_free() / 1e6);
@@ -1339,7 +1345,8 @@ zmc_status plain_prepare(zmc_plan *plan) {
   }
   plan->d_prec = static_cast<double *>(plan->alloc(total * sizeof(double)));
   PlainJob *jobs_dev = static_cast<PlainJob *>(plan->alloc(n * sizeof(PlainJob)));
-  if (!plan->d_prec || !jobs_dev) return set_error(ZMC_ENOMEM, "plain form: arena full");
+  if (!plan->d_prec || !jobs_dev)
+    return ctx->poisoned ? ZMC_ECUDA : set_error(ZMC_ENOMEM, "plain form: arena full");
   std::vector<PlainJob> jobs(n);
   for (size_t i = 0; i < n; ++i) {
     jobs[i].rec = plan->d_prec + plan->poff[i];
@@ -1684,7 +1691,7 @@ zmc_status zmc_philox4x32_10(zmc_ctx *ctx, const uint32_t *ctr, const uint32_t *
   std::lock_guard<std::recursive_mutex> g(ctx->api_mu);
   const size_t bytes = n * 40;  // 16 ctr + 8 key + 16 out
   char *d = static_cast<char *>(arena_take(ctx, bytes));
-  if (!d) return set_error(ZMC_ENOMEM, "arena full");
+  if (!d) return ctx->poisoned ? ZMC_ECUDA : set_error(ZMC_ENOMEM, "arena full");
   st = ensure_stage(ctx, bytes);
   if (st == ZMC_OK) {
     char *s = static_cast<char *>(ctx->stage);
@@ -1720,7 +1727,7 @@ zmc_status zmc_philox_rate(zmc_ctx *ctx, uint64_t n_blocks, double *blocks_per_s
   if (per > 0xFFFFFFF0ull) return set_error(ZMC_EINVAL, "n_blocks too large for one wave");
   const uint32_t per_thread = static_cast<uint32_t>(per);
   uint32_t *d = static_cast<uint32_t *>(arena_take(ctx, threads * sizeof(uint32_t)));
-  if (!d) return set_error(ZMC_ENOMEM, "arena full");
+  if (!d) return ctx->poisoned ? ZMC_ECUDA : set_error(ZMC_ENOMEM, "arena full");
   cudaEvent_t ev[2] = {nullptr, nullptr};
   cudaError_t e = cudaEventCreate(&ev[0]);
   if (e == cudaSuccess) e = cudaEventCreate(&ev[1]);
@@ -1755,7 +1762,7 @@ zmc_status zmc_eval_samples(zmc_ctx *ctx, const zmc_desc *desc, uint64_t s_begin
   std::lock_guard<std::recursive_mutex> g(ctx->api_mu);
   const size_t bytes = sizeof(FnDev) + static_cast<size_t>(count) * 4;
   char *d = static_cast<char *>(arena_take(ctx, bytes));
-  if (!d) return set_error(ZMC_ENOMEM, "arena full");
+  if (!d) return ctx->poisoned ? ZMC_ECUDA : set_error(ZMC_ENOMEM, "arena full");
   st = ensure_stage(ctx, bytes);
   if (st == ZMC_OK) {
     char *s = static_cast<char *>(ctx->stage);

@@ -147,7 +147,8 @@ struct UploadPart {
 };
 cudaError_t upload_parts(const UploadPart *parts, size_t n, const char *stage, cudaStream_t stream);
 // Device memory for a table from the context's arena, taking back the plans' split
-// scratch when there is no room otherwise (under api_mu).
+// scratch when there is no room otherwise (under api_mu).  Null without room, or after
+// a CUDA error there (the context is poisoned and the error text set).
 void *arena_take(zmc_ctx *ctx, size_t bytes);
 // Whether blocks of `bytes` in all could be taken so.  Asked before a table's first
 // block: a table that cannot fit takes no plan's scratch.

@@ -291,6 +291,7 @@ zmc_status udf_run(zmc_ctx *ctx, const zmc_udf *udf, const UdfRow *rows, size_t 
     sorted = sorted && (i == 0 || fns[i - 1].variant <= fns[i].variant);
   }
   const auto no_room = [&] {
+    if (ctx->poisoned) return ZMC_ECUDA;
     return set_error(ZMC_ENOMEM, "udf call needs %.1f MB of device memory",
                      (fn_b + total * 8.0 + n * 64.0 + p_b) / 1e6);
   };

@@ -16,6 +16,7 @@ struct Range {
 };
 std::vector<Range> g_uploads;       // host-to-device copies
 std::vector<std::string> g_events;  // launches and counter resets, in order
+bool g_sync_fails = false;
 
 void note(const char *fmt, ...) {
   char buf[256];
@@ -42,7 +43,9 @@ cudaError_t cudaStreamCreateWithFlags(cudaStream_t *s, unsigned) {
   return *s = reinterpret_cast<cudaStream_t>(std::malloc(1)), cudaSuccess;
 }
 cudaError_t cudaStreamDestroy(cudaStream_t s) { return std::free(s), cudaSuccess; }
-cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaStreamSynchronize(cudaStream_t) {
+  return g_sync_fails ? cudaErrorLaunchFailure : cudaSuccess;
+}
 cudaError_t cudaStreamWaitEvent(cudaStream_t, cudaEvent_t, unsigned) { return cudaSuccess; }
 cudaError_t cudaEventCreate(cudaEvent_t *e) {
   return *e = reinterpret_cast<cudaEvent_t>(std::malloc(1)), cudaSuccess;
@@ -272,6 +275,19 @@ void scratch_taken_from(size_t rows) {
   zmc_destroy(c);
 }
 
+// The wait for a plan's last launches fails while its scratch is taken back.
+void scratch_cannot_be_taken() {
+  zmc_ctx *c = context(table_bytes(1000) + split_bytes(1000, 1000, 104) + 4096, 104);
+  zmc_plan *a = plan(c, unlike_rows(1000)), *b = nullptr;
+  const std::vector<zmc_desc> rows = unlike_rows(1000);
+  g_sync_fails = true;
+  std::printf("%d\n", zmc_plan_create(c, rows.data(), rows.size(), &b));
+  g_sync_fails = false;
+  std::printf("%d\n", zmc_plan_run(a, ZMC_STAGE_ALL));
+  zmc_plan_destroy(a);
+  zmc_destroy(c);
+}
+
 }  // namespace
 
 int main(int, char **argv) {
@@ -282,5 +298,6 @@ int main(int, char **argv) {
   if (what == "two_serving_tables") two_tables(true);
   if (what == "scratch_taken_after_sampling") scratch_taken_after_sampling();
   if (what == "scratch_taken_from") scratch_taken_from(std::strtoul(argv[2], nullptr, 10));
+  if (what == "scratch_cannot_be_taken") scratch_cannot_be_taken();
   return 0;
 }

@@ -6,7 +6,7 @@ import subprocess
 
 import pytest
 
-from paper_2104_10073_gb300 import build
+from paper_2104_10073_gb300 import build, zmc
 
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
@@ -51,3 +51,7 @@ def test_taking_scratch_back_makes_records_and_writes_no_result(run):
 @pytest.mark.parametrize("rows,taken,whole", [(1000, 1, 1), (100000, 0, 0)])
 def test_no_more_scratch_is_taken_back_than_makes_room(run, rows, taken, whole):
     assert run("scratch_taken_from", str(rows)) == [str(taken), str(whole)]
+
+
+def test_a_cuda_error_while_scratch_is_taken_back_is_reported(run):
+    assert run("scratch_cannot_be_taken") == [str(zmc.ZMC_ECUDA)] * 2
