@@ -613,8 +613,12 @@ struct zmc_plan {
   uint64_t n_chunks = 0, n_samples = 0;
   uint64_t fam_items[4] = {0, 0, 0, 0};
   uint64_t fam_units[4] = {0, 0, 0, 0};  // whole chunks and blocks of split ones
-  bool splits = false;        // chunks may be split: the merge is the finish kernel
-  void *d_split = nullptr;    // their scratch
+  // Chunks of each family to split, while there is scratch for it (h_hdr.split then
+  // says the same).  The launches and the finish kernel, which takes the merge's place
+  // (splits), are right with and without it, so a captured graph stays valid.
+  uint32_t split[4] = {0, 0, 0, 0};
+  bool splits = false;
+  void *d_split = nullptr;    // the scratch
   size_t scratch_bytes = 0;   // its size (split_bytes)
   bool dirty = false;          // the counters were drawn from and not reset
   bool ranged = false;  // built by zmc_integrate_moments (no plain form)
@@ -646,9 +650,26 @@ struct zmc_plan {
 
 namespace zmc {
 
+// Scratch for a plan's split chunks, if there is room, and the header with it (on the
+// host: the counts and the device's header are the caller's to write).
+static bool take_scratch(zmc_plan *p) {
+  p->d_split = p->ctx->arena.alloc(p->scratch_bytes);
+  if (!p->d_split) return false;
+  p->ctx->split_plans.insert(p);
+  p->h_hdr.left = static_cast<uint32_t *>(p->d_split);
+  auto *part = reinterpret_cast<float2 *>(static_cast<char *>(p->d_split) +
+                                          round256(p->n * sizeof(uint32_t)));
+  for (int f = 0; f < 4; ++f) {
+    p->h_hdr.split[f] = p->split[f];
+    p->h_hdr.part[f] = part;
+    part += static_cast<size_t>(p->split[f]) * chunk_blocks(p->quints) * 32;
+  }
+  return true;
+}
+
 // Gives plans' scratch back to the arena, of as few plans as make room for `bytes`, of
-// none when all of it would not: from the next run on, those plans hand out whole
-// chunks only.
+// none when all of it would not: those plans hand out whole chunks only until a run
+// of theirs finds room again.
 static void drop_splits(zmc_ctx *ctx, size_t bytes) {
   std::vector<zmc_plan *> drop(ctx->split_plans.begin(), ctx->split_plans.end());
   const auto fits = [&](const zmc_plan *but) {
@@ -1106,7 +1127,8 @@ zmc_status plan_build(zmc_ctx *ctx, const zmc_desc *desc, size_t n, zmc_plan **o
   // chunks of each family and how many of them are split
   uint64_t fam_chunks[4] = {0, 0, 0, 0};
   for (size_t i = 0; i < n; ++i) fam_chunks[desc[i].family] += nchunk[i];
-  uint32_t dmin = kMaxDim, dmax = 1, split[4], n_split = 0;
+  uint32_t dmin = kMaxDim, dmax = 1, n_split = 0;
+  uint32_t *split = plan->split;
   bool alike = true;  // one family, one degree, dimensions within a factor 3/2
   for (size_t i = 0; i < n; ++i) {
     dmin = std::min(dmin, desc[i].dim);
@@ -1193,25 +1215,17 @@ zmc_status plan_build(zmc_ctx *ctx, const zmc_desc *desc, size_t n, zmc_plan **o
   // room for it every chunk stays whole (arena_take takes it back when a later
   // table needs the room; the serving scheduler cannot, so a plan of a serving
   // context that outlives the call has none)
-  if (n_split && !(ctx->serving && keep))
-    plan->d_split = ctx->arena.alloc(split_bytes(n, n_split, plan->quints));
-  if (plan->d_split) {
+  plan->splits = n_split && !(ctx->serving && keep);
+  if (plan->splits) {
     plan->scratch_bytes = split_bytes(n, n_split, plan->quints);
-    plan->splits = true;
-    ctx->split_plans.insert(plan.get());
-    h.left = static_cast<uint32_t *>(plan->d_split);
-    auto *part = reinterpret_cast<float2 *>(static_cast<char *>(plan->d_split) +
-                                            round256(n * sizeof(uint32_t)));
-    for (int f = 0; f < 4; ++f) {
-      h.split[f] = split[f];
-      h.part[f] = part;
-      part += static_cast<size_t>(split[f]) * chunk_blocks(plan->quints) * 32;
-    }
+    take_scratch(plan.get());
+  } else {
+    std::fill(split, split + 4, 0u);
   }
   for (int f = 0; f < 4; ++f) {
     const int unroll = static_cast<int>(plan->unroll[f]);
     plan->fam_items[f] = h.item_end[f] - h.item_begin[f];
-    plan->fam_units[f] = launch_units(plan->fam_items[f], h.split[f], plan->quints);
+    plan->fam_units[f] = launch_units(plan->fam_items[f], split[f], plan->quints);
     plan->block[f] = spread_block(ctx->shape.block, plan->fam_units[f], ctx->sms);
     plan->grid[f] = grid_for(ctx, f, plan->block[f], ctx->shape.blocks_per_sm[f],
                              plan->fam_units[f], unroll);
@@ -1269,6 +1283,18 @@ zmc_status plan_reset(zmc_plan *plan) {
   return ZMC_OK;
 }
 
+// A plan without its scratch takes it again when there is room: what it lost to a table
+// that has gone since would slow all of its later runs down.
+zmc_status plan_regain(zmc_plan *plan) {
+  if (!plan->splits || plan->d_split || !take_scratch(plan)) return ZMC_OK;
+  zmc_ctx *ctx = plan->ctx;
+  ZMC_CUDA(ctx, cudaMemsetAsync(plan->h_hdr.left, 0, plan->n * sizeof(uint32_t), ctx->stream));
+  ZMC_CUDA(ctx, cudaMemcpyAsync(plan->d_hdr, &plan->h_hdr, sizeof plan->h_hdr,
+                                cudaMemcpyHostToDevice, ctx->stream));
+  plan->dirty = false;
+  return ZMC_OK;
+}
+
 zmc_status plan_enqueue(zmc_plan *plan, uint32_t stages) {
   zmc_ctx *ctx = plan->ctx;
   cudaStream_t str = ctx->stream;
@@ -1284,7 +1310,7 @@ zmc_status plan_enqueue(zmc_plan *plan, uint32_t stages) {
   if (stages & ZMC_STAGE_MERGE) {
     if (plan->splits) {  // also after the scratch went: then every row merges at once
       uint64_t warps = plan->n;
-      for (uint32_t k : plan->h_hdr.split) warps += k;
+      for (uint32_t k : plan->split) warps += k;
       ZMC_CUDA(ctx, launch_finish(plan->d_entries, plan->d_hdr, warps, ctx->sms, str));
     } else {
       const unsigned grid = static_cast<unsigned>(
@@ -1538,6 +1564,8 @@ zmc_status zmc_plan_run(zmc_plan *plan, uint32_t stages) {
     return set_error(ZMC_EINVAL, "stages must be a non-empty subset of ZMC_STAGE_ALL");
   std::lock_guard<std::recursive_mutex> g(ctx->api_mu);
   if (stages != ZMC_STAGE_ALL) return plan_enqueue(plan, stages);
+  st = plan_regain(plan);
+  if (st != ZMC_OK) return st;
   st = plan_reset(plan);  // outside the graph, which is captured with clean counters
   if (st != ZMC_OK) return st;
   if (!plan->graph) {

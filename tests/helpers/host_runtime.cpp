@@ -288,6 +288,22 @@ void scratch_cannot_be_taken() {
   zmc_destroy(c);
 }
 
+// Split chunks of a plan at first, with its scratch taken, and run again after the table
+// that took it has gone.
+void scratch_comes_back() {
+  zmc_ctx *c = context(table_bytes(1000) + split_bytes(1000, 1000, 104) + 4096, 104);
+  zmc_plan *a = plan(c, unlike_rows(1000));
+  std::printf("%u", split_of(a));
+  zmc_plan *b = plan(c, unlike_rows(1000));
+  zmc_plan_run(a, ZMC_STAGE_ALL);
+  std::printf(" %u", split_of(a));
+  zmc_plan_destroy(b);
+  zmc_plan_run(a, ZMC_STAGE_ALL);
+  std::printf(" %u\n", split_of(a));
+  zmc_plan_destroy(a);
+  zmc_destroy(c);
+}
+
 }  // namespace
 
 int main(int, char **argv) {
@@ -299,5 +315,6 @@ int main(int, char **argv) {
   if (what == "scratch_taken_after_sampling") scratch_taken_after_sampling();
   if (what == "scratch_taken_from") scratch_taken_from(std::strtoul(argv[2], nullptr, 10));
   if (what == "scratch_cannot_be_taken") scratch_cannot_be_taken();
+  if (what == "scratch_comes_back") scratch_comes_back();
   return 0;
 }

@@ -55,3 +55,7 @@ def test_no_more_scratch_is_taken_back_than_makes_room(run, rows, taken, whole):
 
 def test_a_cuda_error_while_scratch_is_taken_back_is_reported(run):
     assert run("scratch_cannot_be_taken") == [str(zmc.ZMC_ECUDA)] * 2
+
+
+def test_scratch_comes_back_when_there_is_room_again(run):
+    assert run("scratch_comes_back") == ["1000 0 1000"]
