@@ -621,6 +621,9 @@ struct zmc_plan {
   void *d_split = nullptr;    // the scratch
   size_t scratch_bytes = 0;   // its size (split_bytes)
   bool dirty = false;          // the counters were drawn from and not reset
+  // A caller captured a run of this plan into a graph of its own: it may replay any
+  // time, so nothing is known of the counters or of unmerged samples from here on.
+  bool captured = false;
   bool ranged = false;  // built by zmc_integrate_moments (no plain form)
   uint32_t quints = 0;  // chunk = 160 * quints samples
   unsigned unroll[4] = {1, 1, 1, 1};  // quint-loop unroll of each family kernel
@@ -649,6 +652,13 @@ struct zmc_plan {
 };
 
 namespace zmc {
+
+// Whether the caller captures the context's stream into a graph of its own.
+static bool capturing(const zmc_ctx *ctx) {
+  cudaStreamCaptureStatus s = cudaStreamCaptureStatusNone;
+  return cudaStreamIsCapturing(ctx->stream, &s) == cudaSuccess &&
+         s == cudaStreamCaptureStatusActive;
+}
 
 // Scratch for a plan's split chunks, if there is room, and the header with it (on the
 // host: the counts and the device's header are the caller's to write).
@@ -683,7 +693,8 @@ static void drop_splits(zmc_ctx *ctx, size_t bytes) {
     if (fits(drop[k])) drop.erase(drop.begin() + static_cast<ptrdiff_t>(k));
   cudaError_t e = cudaSuccess;
   for (zmc_plan *p : drop) {
-    if (e == cudaSuccess && p->dirty) {
+    if (e == cudaSuccess && p->captured) e = cudaDeviceSynchronize();  // its replays
+    if (e == cudaSuccess && (p->dirty || p->captured)) {
       // sampled, not merged yet: the records are still to be made (a merge that nobody
       // asked for would write over the plan's results)
       uint64_t warps = p->n;
@@ -711,7 +722,7 @@ static void drop_splits(zmc_ctx *ctx, size_t bytes) {
 
 void *arena_take(zmc_ctx *ctx, size_t bytes) {
   void *p = ctx->arena.alloc(bytes);
-  if (!p && !ctx->split_plans.empty()) {
+  if (!p && !ctx->split_plans.empty() && !capturing(ctx)) {  // it waits for the stream
     drop_splits(ctx, bytes);
     p = ctx->arena.alloc(bytes);
   }
@@ -1274,9 +1285,9 @@ zmc_status plan_build(zmc_ctx *ctx, const zmc_desc *desc, size_t n, zmc_plan **o
 }
 
 // The counters are zero after the upload and after each merge; a sampling stage run
-// by itself leaves them drawn from.
+// by itself leaves them drawn from, and so may a replay of a caller's graph.
 zmc_status plan_reset(zmc_plan *plan) {
-  if (!plan->dirty) return ZMC_OK;
+  if (!plan->dirty && !plan->captured) return ZMC_OK;
   ZMC_CUDA(plan->ctx, cudaMemsetAsync(plan->d_hdr, 0, sizeof(plan->d_hdr->counter),
                                       plan->ctx->stream));
   plan->dirty = false;
@@ -1563,8 +1574,10 @@ zmc_status zmc_plan_run(zmc_plan *plan, uint32_t stages) {
   if ((stages & ZMC_STAGE_ALL) == 0 || (stages & ~ZMC_STAGE_ALL))
     return set_error(ZMC_EINVAL, "stages must be a non-empty subset of ZMC_STAGE_ALL");
   std::lock_guard<std::recursive_mutex> g(ctx->api_mu);
+  const bool in_capture = capturing(ctx);
+  if (in_capture) plan->captured = true;
   if (stages != ZMC_STAGE_ALL) return plan_enqueue(plan, stages);
-  st = plan_regain(plan);
+  st = in_capture ? ZMC_OK : plan_regain(plan);
   if (st != ZMC_OK) return st;
   st = plan_reset(plan);  // outside the graph, which is captured with clean counters
   if (st != ZMC_OK) return st;

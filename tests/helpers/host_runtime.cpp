@@ -17,6 +17,7 @@ struct Range {
 std::vector<Range> g_uploads;       // host-to-device copies
 std::vector<std::string> g_events;  // launches and counter resets, in order
 bool g_sync_fails = false;
+bool g_capturing = false;  // a caller's capture
 
 void note(const char *fmt, ...) {
   char buf[256];
@@ -70,6 +71,14 @@ cudaError_t cudaMemcpyAsync(void *to, const void *from, size_t n, cudaMemcpyKind
 cudaError_t cudaMemsetAsync(void *to, int v, size_t n, cudaStream_t) {
   note("memset");
   std::memset(to, v, n);
+  return cudaSuccess;
+}
+cudaError_t cudaDeviceSynchronize() {
+  note("device sync");
+  return cudaSuccess;
+}
+cudaError_t cudaStreamIsCapturing(cudaStream_t, cudaStreamCaptureStatus *s) {
+  *s = g_capturing ? cudaStreamCaptureStatusActive : cudaStreamCaptureStatusNone;
   return cudaSuccess;
 }
 cudaError_t cudaStreamBeginCapture(cudaStream_t, cudaStreamCaptureMode) { return cudaSuccess; }
@@ -304,6 +313,32 @@ void scratch_comes_back() {
   zmc_destroy(c);
 }
 
+// What a caller's graph of the sampling stage holds, what a run holds after that graph
+// may have been replayed, and what taking the scratch back then does.
+void captured_by_a_caller() {
+  zmc_ctx *c = context(table_bytes(1000) + split_bytes(1000, 1000, 104) + 4096, 104);
+  zmc_plan *a = plan(c, unlike_rows(1000)), *b;
+  const auto run = [&](uint32_t stages) {
+    g_events.clear();
+    zmc_plan_run(a, stages);
+    for (const std::string &e : g_events) std::printf("%s; ", e.c_str());
+    std::printf("\n");
+  };
+  g_capturing = true;
+  run(ZMC_STAGE_SAMPLE);
+  g_capturing = false;
+  run(ZMC_STAGE_MERGE);
+  run(ZMC_STAGE_SAMPLE);
+  zmc_plan_run(a, ZMC_STAGE_MERGE);
+  g_events.clear();
+  b = plan(c, unlike_rows(1000));
+  for (const std::string &e : g_events) std::printf("%s; ", e.c_str());
+  std::printf("\n");
+  zmc_plan_destroy(a);
+  zmc_plan_destroy(b);
+  zmc_destroy(c);
+}
+
 }  // namespace
 
 int main(int, char **argv) {
@@ -316,5 +351,6 @@ int main(int, char **argv) {
   if (what == "scratch_taken_from") scratch_taken_from(std::strtoul(argv[2], nullptr, 10));
   if (what == "scratch_cannot_be_taken") scratch_cannot_be_taken();
   if (what == "scratch_comes_back") scratch_comes_back();
+  if (what == "captured_by_a_caller") captured_by_a_caller();
   return 0;
 }

@@ -59,3 +59,11 @@ def test_a_cuda_error_while_scratch_is_taken_back_is_reported(run):
 
 def test_scratch_comes_back_when_there_is_room_again(run):
     assert run("scratch_comes_back") == ["1000 0 1000"]
+
+
+def test_a_callers_graph_of_the_sampling_stage_resets_the_counters(run):
+    assert run("captured_by_a_caller") == [
+        "memset; batched 2 split 1000; ",
+        "finish split 1000; ",
+        "memset; batched 2 split 1000; ",  # the graph may have been replayed in between
+        "device sync; records split 1000; "]
