@@ -751,6 +751,11 @@ zmc_status check_ctx(zmc_ctx *ctx) {
 // block, resident blocks per SM) that runs a bounded slice of the plan's own
 // items fastest, or the cached choice for the same key.  Geometry never changes
 // results; the slice's records are recomputed identically by the real launch.
+// A launch of fewer units (chunks and blocks of split ones) than the chip keeps warps
+// keeps the geometry plan_build gave it: that spreads the units over the SMs (56 units
+// in as many one-warp blocks, where a choice made on a large table would put them into
+// 14 of four warps), and all geometries take it in one wave, so that timing them would
+// put noise into the cache.
 zmc_status plan_autotune(zmc_plan *plan) {
   zmc_ctx *ctx = plan->ctx;
   cudaStream_t str = ctx->stream;
@@ -759,6 +764,9 @@ zmc_status plan_autotune(zmc_plan *plan) {
   for (int f = 0; f < 4 && st == ZMC_OK; ++f) {
     if (plan->fam_items[f] == 0) continue;
     const int U = static_cast<int>(plan->unroll[f]);
+    const uint64_t warps = static_cast<uint64_t>(ctx->sms) * 8 *
+                           std::max(batched_max_blocks_per_sm(f, 256, U), 1);
+    if (plan->fam_units[f] < warps) continue;
     const std::string key = tune_key(ctx, f, plan->dominant_dim[f], plan->quints, U);
     auto hit = ctx->tune_cache.find(key);
     if (hit != ctx->tune_cache.end()) {
@@ -785,12 +793,14 @@ zmc_status plan_autotune(zmc_plan *plan) {
       th.split[g] = 0;
     }
     th.item_end[f] = th.item_begin[f] + slice;
+    if (slice == plan->fam_items[f]) th.split[f] = plan->h_hdr.split[f];  // as it will run
+    const uint64_t units = launch_units(slice, th.split[f], plan->quints);
     TuneChoice best;
     best.ms = 1e30f;
     for (unsigned block : {128u, 256u}) {
       const int maxb = batched_max_blocks_per_sm(f, static_cast<int>(block), U);
       for (int bps = 1; bps <= maxb && st == ZMC_OK; ++bps) {
-        const unsigned grid = grid_for(ctx, f, block, static_cast<unsigned>(bps), slice, U);
+        const unsigned grid = grid_for(ctx, f, block, static_cast<unsigned>(bps), units, U);
         float ms_best = 1e30f;
         for (int rep = 0; rep < 3; ++rep) {
           cudaError_t e = cudaMemcpyAsync(plan->d_hdr, &th, sizeof th, cudaMemcpyHostToDevice, str);

@@ -339,6 +339,29 @@ void captured_by_a_caller() {
   zmc_destroy(c);
 }
 
+// With the geometry tuner: what it times for a table of 3000 chunks, and the launch of
+// one row after it.
+void tuned_geometry() {
+  zmc_options o;
+  zmc_default_options(&o);
+  o.mem_budget_bytes = 64 << 20;
+  o.quints_per_lane = 104;
+  o.autotune = ZMC_TUNE_GEOMETRY;
+  zmc_ctx *c = nullptr;
+  if (zmc_create(&o, &c) != ZMC_OK) std::abort();
+  zmc_plan *a = plan(c, unlike_rows(3000));
+  std::printf("%s\n", g_events.empty() ? "nothing" : g_events[0].c_str());
+  g_events.clear();
+  zmc_plan *b = plan(c, gauss_rows(1, 1, 100000));
+  zmc_plan_info i;
+  zmc_plan_info_get(b, &i);
+  std::printf("%zu %u %u %d\n", g_events.size(), i.family_grid[2], i.family_block[2],
+              i.tune_source[2]);
+  zmc_plan_destroy(a);
+  zmc_plan_destroy(b);
+  zmc_destroy(c);
+}
+
 }  // namespace
 
 int main(int, char **argv) {
@@ -352,5 +375,6 @@ int main(int, char **argv) {
   if (what == "scratch_cannot_be_taken") scratch_cannot_be_taken();
   if (what == "scratch_comes_back") scratch_comes_back();
   if (what == "captured_by_a_caller") captured_by_a_caller();
+  if (what == "tuned_geometry") tuned_geometry();
   return 0;
 }

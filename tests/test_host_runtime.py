@@ -67,3 +67,8 @@ def test_a_callers_graph_of_the_sampling_stage_resets_the_counters(run):
         "finish split 1000; ",
         "memset; batched 2 split 1000; ",  # the graph may have been replayed in between
         "device sync; records split 1000; "]
+
+
+def test_geometry_tuner_times_what_runs_and_leaves_small_launches_spread(run):
+    # one row of 7 chunks, the last of 160 samples: 56 units, one warp per block and SM
+    assert run("tuned_geometry") == ["batched 2 split 2432", "0 56 32 0"]
