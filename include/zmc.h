@@ -192,7 +192,8 @@ typedef struct zmc_plan_info {
     uint32_t family_unroll[4]; /* quint-loop unroll of each family kernel (1 or 2)  */
     int32_t chunk_tune_source; /* chunk length and unroll: 0 default (quints_per_lane
                                   of the context, unroll 1), 1 measured, 2 cached   */
-    uint32_t reserved;
+    uint32_t split_chunks;     /* chunks handed out by accumulation blocks now: 0 while
+                                  there is no room for their scratch                */
 } zmc_plan_info;
 
 typedef struct zmc_serving_stats {

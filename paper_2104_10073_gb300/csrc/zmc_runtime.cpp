@@ -1649,7 +1649,8 @@ zmc_status zmc_plan_info_get(const zmc_plan *plan, zmc_plan_info *out) {
   out->sms = static_cast<uint32_t>(plan->ctx->sms);
   for (int f = 0; f < 4; ++f) out->family_unroll[f] = plan->unroll[f];
   out->chunk_tune_source = plan->chunk_source;
-  out->reserved = 0;
+  out->split_chunks = 0;
+  for (uint32_t k : plan->h_hdr.split) out->split_chunks += k;
   return ZMC_OK;
 }
 

@@ -58,7 +58,7 @@ class zmc_plan_info(ctypes.Structure):
                 ("sms", ctypes.c_uint32), ("family_grid", ctypes.c_uint32 * 4),
                 ("family_block", ctypes.c_uint32 * 4), ("tune_source", ctypes.c_int32 * 4),
                 ("family_unroll", ctypes.c_uint32 * 4), ("chunk_tune_source", ctypes.c_int32),
-                ("reserved", ctypes.c_uint32)]
+                ("split_chunks", ctypes.c_uint32)]
 
 
 class zmc_normal_opts(ctypes.Structure):
