@@ -751,28 +751,28 @@ zmc_status check_ctx(zmc_ctx *ctx) {
 // block, resident blocks per SM) that runs a bounded slice of the plan's own
 // items fastest, or the cached choice for the same key.  Geometry never changes
 // results; the slice's records are recomputed identically by the real launch.
-// A launch of fewer units (chunks and blocks of split ones) than the chip keeps warps
-// keeps the geometry plan_build gave it: that spreads the units over the SMs (56 units
-// in as many one-warp blocks, where a choice made on a large table would put them into
-// 14 of four warps), and all geometries take it in one wave, so that timing them would
-// put noise into the cache.
+// The choice may stem from a larger table (the key names no size) and says nothing of
+// launches whose units (chunks and blocks of split ones) do not fill a block on every
+// SM: those are spread as plan_build spreads them (56 units in as many one-warp blocks,
+// where the choice alone would put them into 14 of four warps).
 zmc_status plan_autotune(zmc_plan *plan) {
   zmc_ctx *ctx = plan->ctx;
   cudaStream_t str = ctx->stream;
   cudaEvent_t e0 = nullptr, e1 = nullptr;  // created at the first cache miss
   zmc_status st = ZMC_OK;
+  const auto shape = [&](int f, const TuneChoice &c) {
+    plan->block[f] = spread_block(c.block, plan->fam_units[f], ctx->sms);
+    plan->grid[f] = grid_for(ctx, f, plan->block[f],
+                             plan->block[f] == c.block ? c.blocks_per_sm : 0, plan->fam_units[f],
+                             static_cast<int>(plan->unroll[f]));
+  };
   for (int f = 0; f < 4 && st == ZMC_OK; ++f) {
     if (plan->fam_items[f] == 0) continue;
     const int U = static_cast<int>(plan->unroll[f]);
-    const uint64_t warps = static_cast<uint64_t>(ctx->sms) * 8 *
-                           std::max(batched_max_blocks_per_sm(f, 256, U), 1);
-    if (plan->fam_units[f] < warps) continue;
     const std::string key = tune_key(ctx, f, plan->dominant_dim[f], plan->quints, U);
     auto hit = ctx->tune_cache.find(key);
     if (hit != ctx->tune_cache.end()) {
-      plan->block[f] = hit->second.block;
-      plan->grid[f] = grid_for(ctx, f, hit->second.block, hit->second.blocks_per_sm,
-                               plan->fam_units[f], U);
+      shape(f, hit->second);
       plan->tune_source[f] = 2;
       continue;
     }
@@ -825,8 +825,7 @@ zmc_status plan_autotune(zmc_plan *plan) {
       }
     }
     if (st != ZMC_OK) break;
-    plan->block[f] = best.block;
-    plan->grid[f] = grid_for(ctx, f, best.block, best.blocks_per_sm, plan->fam_units[f], U);
+    shape(f, best);
     plan->tune_source[f] = 1;
     tune_cache_store(ctx, key, best);
   }

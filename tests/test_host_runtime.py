@@ -71,4 +71,4 @@ def test_a_callers_graph_of_the_sampling_stage_resets_the_counters(run):
 
 def test_geometry_tuner_times_what_runs_and_leaves_small_launches_spread(run):
     # one row of 7 chunks, the last of 160 samples: 56 units, one warp per block and SM
-    assert run("tuned_geometry") == ["batched 2 split 2432", "0 56 32 0"]
+    assert run("tuned_geometry") == ["batched 2 split 2432", "0 56 32 2"]
