@@ -362,6 +362,37 @@ void tuned_geometry() {
   zmc_destroy(c);
 }
 
+// Of each table the chunks that its plan splits.
+void split_rule() {
+  zmc_ctx *c = context(64 << 20, 104);
+  const auto of = [&](const std::vector<zmc_desc> &rows) {
+    zmc_plan *p = plan(c, rows);
+    zmc_plan_info i;
+    zmc_plan_info_get(p, &i);
+    zmc_plan_destroy(p);
+    return i.split_chunks;
+  };
+  const auto alike = [&](uint32_t dim, std::initializer_list<int> counts) {
+    for (int n : counts) std::printf("%u ", of(gauss_rows(n, dim, 1)));
+    std::printf("\n");
+  };
+  alike(1, {1, 851, 852, 1216, 1217, 1629, 1630, 2432, 2433, 9000});
+  alike(3, {1, 972, 973, 1216, 1217, 1945, 1946, 2432, 2433, 9000});
+  for (int n : {2433, 3404, 3405, 3648, 3649, 4864, 4865})  // whole chunks: 1 to 2 waves
+    std::printf("%u ", of(gauss_rows(n, 3, 16640)));
+  // 2800 chunks of 0.99 and 0.79 waves of work
+  std::printf("%u %u\n", of(gauss_rows(400, 3, 100000)), of(gauss_rows(2800, 3, 11400)));
+  std::vector<zmc_desc> rows = gauss_rows(3000, 2, 1);  // two and three dimensions: alike
+  for (size_t i = 0; i < rows.size(); i += 2) rows[i] = gauss_rows(1, 3, 1)[0];
+  std::printf("%u %u %u ", of(rows), of(unlike_rows(2000)), of(unlike_rows(3000)));
+  for (zmc_desc &d : rows) {  // constants
+    d.family = ZMC_POLY;
+    d.deg = 0;
+  }
+  std::printf("%u\n", of(rows));
+  zmc_destroy(c);
+}
+
 }  // namespace
 
 int main(int, char **argv) {
@@ -376,5 +407,6 @@ int main(int, char **argv) {
   if (what == "scratch_comes_back") scratch_comes_back();
   if (what == "captured_by_a_caller") captured_by_a_caller();
   if (what == "tuned_geometry") tuned_geometry();
+  if (what == "split_rule") split_rule();
   return 0;
 }

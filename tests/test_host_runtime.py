@@ -72,3 +72,13 @@ def test_a_callers_graph_of_the_sampling_stage_resets_the_counters(run):
 def test_geometry_tuner_times_what_runs_and_leaves_small_launches_spread(run):
     # one row of 7 chunks, the last of 160 samples: 56 units, one warp per block and SM
     assert run("tuned_geometry") == ["batched 2 split 2432", "0 56 32 2"]
+
+
+def test_split_rule(run):
+    """Resident warps 2432: nothing beyond the lines near two and four warps per scheduler,
+    half a wave of equal chunks above one unless the work ends on two warps per scheduler
+    or fits one wave, a wave of unlike ones, and no constant."""
+    assert run("split_rule") == ["1 851 0 0 1217 1629 0 0 1216 1216 ",
+                                 "1 972 0 0 1217 1945 0 0 1216 1216 ",
+                                 "1216 1216 0 0 1216 1216 1216 0 1216",
+                                 "0 2000 2432 0"]
