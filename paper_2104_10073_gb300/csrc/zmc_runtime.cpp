@@ -517,20 +517,46 @@ unsigned family_grid(const zmc_ctx *ctx, int family, uint64_t items, int unroll)
 // against 92 us.  A block costs its draw, lookup and descriptor loads again, ~2.5 us
 // of latency, so chunks that are alike and nearly fill a whole number of warps per
 // scheduler stay whole (1216 chunks, two warps: 54 against 62 us; 2432, four: 93
-// against 110), and so do alike chunks in more than one wave, which end together
-// anyway (4864: 171 either way, 188 split).
+// against 110).  The lines, in parts of a wave (W = 2432 warps), where whole chunks
+// begin to win: 0.8 W for four warps (3-D abs-linear at 0.79: 84 split, 88 whole) and
+// 2/3 W in one dimension, whose chunks are short (0.70 / 0.77: abs-linear 49.3 / 53.4
+// split, 48 whole; degree-1 polynomials 51.3 / 53.4 and 47.5); 0.4 W for two warps, and
+// 0.35 W in one and two dimensions (0.39: 1-D abs-linear 32.9 and 29, 2-D polynomials
+// 43 and 39).  A constant (a polynomial of degree 0) draws nothing, and its chunks,
+// 26 us a wave, are never worth splitting (0.8 W: 39 split).
+// Chunks in more than one wave end together only by luck, also when they are alike: the
+// warps of a scheduler do not run evenly, a chunk that starts late runs on alone, and a
+// change of a few instructions anywhere moves the point (4620 Gaussian chunks in 3-D 241
+// and 281 us for two builds of the same loop).  Half a wave by blocks evens the end out
+// where all chunks cost the same, but for work that ends on two warps per scheduler (a
+// last wave of 0.4 to 0.5, where it costs 1 to 5% more often than it helps) and work
+// that fits one wave (400 rows of 10^5 samples, 0.99: 10 to 16% slower).  Over 28 kernels
+// and 25 sizes from 1.02 to 25 waves of work the time is 0.946 of that of whole chunks
+// in the geometric mean (1.02 waves 0.83, 1.3 0.94, 1.7 0.89, 1.9 0.97, 3.7 0.96, 8.5
+// 0.99), at worst 1.07, and 227 us for the 4620 chunks.  A quarter and a whole wave
+// measured slower.  Two dimensions (the Eq. 2 set, 2.5 waves: a call 207 us whole, 215
+// so) and user code (sincosf in FP32, 2.5 waves: 374 and 385) stay whole.
 // Chunks that differ in cost (families, dimensions, polynomial degrees) leave a tail
 // of up to the longest chunk's time at the end and a CTA's slowest warp's time at
 // each change of family: one chunk per resident warp fills it (300 mixed rows 1107
 // against 1295 us, 64 mixed rows 271 against 386).
 // The lane summaries take 256 bytes a block, at most kSplitBytes a family (5 MB at
 // the default Q = 104).  None for chunks of one block.
-uint32_t split_chunks(uint64_t items, bool alike, uint64_t resident_warps, uint32_t quints) {
+uint32_t split_chunks(uint64_t items, uint64_t samples, Chunks chunks, unsigned dim,
+                      uint64_t resident_warps, uint32_t quints) {
   const uint64_t nb = chunk_blocks(quints), w = resident_warps;
-  if (nb < 2) return 0;
-  const bool fills = 5 * items > 4 * w || (5 * items > 2 * w && 2 * items <= w);
-  if (alike && fills) return 0;
-  return static_cast<uint32_t>(std::min({items, w, kSplitBytes / (nb * kPartBytes)}));
+  if (nb < 2 || dim == 0) return 0;
+  const uint64_t most = std::min({items, w, kSplitBytes / (nb * kPartBytes)});
+  if (chunks == Chunks::kEqual && items > w) {
+    const double waves = static_cast<double>(samples) /
+                         (static_cast<double>(chunk_samples_of(quints)) * static_cast<double>(w));
+    const double last = waves - std::floor(waves);
+    const bool even = (last > 0.4 && last <= 0.5) || (waves > 0.8 && waves <= 1.0);
+    return even ? 0u : static_cast<uint32_t>(std::min(most, w / 2));
+  }
+  const uint64_t two = dim <= 2 ? 35 : 40, four = dim <= 1 ? 67 : 80;  // % of w
+  const bool fills = 100 * items > four * w || (100 * items > two * w && 2 * items <= w);
+  return chunks != Chunks::kUnlike && fills ? 0u : static_cast<uint32_t>(most);
 }
 
 // Whole chunks and blocks of split ones.
@@ -1147,19 +1173,22 @@ zmc_status plan_build(zmc_ctx *ctx, const zmc_desc *desc, size_t n, zmc_plan **o
   // chunks of each family and how many of them are split
   uint64_t fam_chunks[4] = {0, 0, 0, 0};
   for (size_t i = 0; i < n; ++i) fam_chunks[desc[i].family] += nchunk[i];
-  uint32_t dmin = kMaxDim, dmax = 1, n_split = 0;
+  uint32_t dmin = kMaxDim, dmax = 0, n_split = 0;  // of the coordinates that are drawn
   uint32_t *split = plan->split;
   bool alike = true;  // one family, one degree, dimensions within a factor 3/2
   for (size_t i = 0; i < n; ++i) {
-    dmin = std::min(dmin, desc[i].dim);
-    dmax = std::max(dmax, desc[i].dim);
-    alike = alike && desc[i].family == desc[0].family &&
-            (desc[i].family != ZMC_POLY || desc[i].deg == desc[0].deg);
+    const bool poly = desc[i].family == ZMC_POLY;
+    const uint32_t d = poly && desc[i].deg == 0 ? 0 : desc[i].dim;
+    dmin = std::min(dmin, d);
+    dmax = std::max(dmax, d);
+    alike = alike && desc[i].family == desc[0].family && (!poly || desc[i].deg == desc[0].deg);
   }
-  alike = alike && 2 * dmax <= 3 * dmin;
+  const Chunks chunks = !alike || 2 * dmax > 3 * dmin ? Chunks::kUnlike
+                        : dmin == dmax                ? Chunks::kEqual
+                                                      : Chunks::kAlike;
   for (int f = 0; f < 4; ++f) {
     const int bps = batched_max_blocks_per_sm(f, 256, static_cast<int>(plan->unroll[f]));
-    split[f] = split_chunks(fam_chunks[f], alike,
+    split[f] = split_chunks(fam_chunks[f], samples, chunks, dmax,
                             static_cast<uint64_t>(ctx->sms) * 8 * std::max(bps, 1), plan->quints);
     n_split += split[f];
   }

@@ -153,7 +153,9 @@ void *arena_take(zmc_ctx *ctx, size_t bytes);
 // Whether blocks of `bytes` in all could be taken so.  Asked before a table's first
 // block: a table that cannot fit takes no plan's scratch.
 bool arena_could_hold(const zmc_ctx *ctx, size_t bytes);
-// Chunks that are handed out by accumulation blocks (LaunchHdr::split).
+// Chunks that are handed out by accumulation blocks (LaunchHdr::split), by how their
+// costs compare, their samples and the most coordinates that one of those draws.
+enum class Chunks { kUnlike, kAlike, kEqual };
 constexpr size_t kPartBytes = 32 * sizeof(float2);  // the lane summaries of one block
 constexpr uint64_t kSplitBytes = 8u << 20;          // at most, per family
 // Scratch of a launch that splits chunks: the finish kernel's counts (a word per row),
@@ -161,7 +163,8 @@ constexpr uint64_t kSplitBytes = 8u << 20;          // at most, per family
 constexpr size_t split_bytes(size_t rows, size_t split, uint32_t quints) {
   return round256(rows * sizeof(uint32_t)) + split * chunk_blocks(quints) * kPartBytes;
 }
-uint32_t split_chunks(uint64_t items, bool alike, uint64_t resident_warps, uint32_t quints);
+uint32_t split_chunks(uint64_t items, uint64_t samples, Chunks chunks, unsigned dim,
+                      uint64_t resident_warps, uint32_t quints);
 uint64_t launch_units(uint64_t items, uint32_t split, uint32_t quints);
 unsigned spread_block(unsigned block, uint64_t units, int sms);
 std::string tune_key(const zmc_ctx *ctx, int family, int dim, uint32_t quints, int unroll);

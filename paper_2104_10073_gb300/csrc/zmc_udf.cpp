@@ -305,7 +305,10 @@ zmc_status udf_run(zmc_ctx *ctx, const zmc_udf *udf, const UdfRow *rows, size_t 
   auto *d_ent = static_cast<Entry *>(ab.get(ent_b));
   auto *d_mrg = static_cast<const FnDev **>(ab.get(mrg_b));
   const uint64_t resident = static_cast<uint64_t>(ctx->sms) * udf->max_blocks * 8;
-  uint32_t split = split_chunks(total, alike, resident, ctx->quints_per_lane);
+  uint32_t dim = 0;
+  for (size_t i = 0; i < n; ++i) dim = std::max(dim, rows[i].dim);
+  uint32_t split = split_chunks(total, 0, alike ? Chunks::kAlike : Chunks::kUnlike, dim, resident,
+                                ctx->quints_per_lane);
   auto *d_hdr = static_cast<LaunchHdr *>(ab.get(sizeof(LaunchHdr)));
   auto *d_p = static_cast<double *>(p_b ? ab.get(p_b) : nullptr);
   if (!d_fns || !d_rec || !d_ent || !d_mrg || !d_hdr || (p_b && !d_p))
