@@ -325,11 +325,15 @@ zmc_status zmc_serving_stats_get(zmc_ctx *ctx, zmc_serving_stats *out);
  * merge launches can be replayed (as a CUDA graph) without host traffic. */
 zmc_status zmc_plan_create(zmc_ctx *ctx, const zmc_desc *desc, size_t n, zmc_plan **out);
 
-#define ZMC_STAGE_SAMPLE 1u /* reset the work counter + persistent sampling launch */
-#define ZMC_STAGE_MERGE 2u  /* FP64 merge of every integrand's chunk records       */
-#define ZMC_STAGE_ALL 3u    /* both, replayed as one captured CUDA graph           */
+#define ZMC_STAGE_SAMPLE 1u /* persistent sampling launch; resets the work counters
+                               first when no merge has done so since the last one   */
+#define ZMC_STAGE_MERGE 2u  /* FP64 merge of every integrand's chunk records (made
+                               first for split chunks); resets the work counters    */
+#define ZMC_STAGE_ALL 3u    /* both, replayed as one captured CUDA graph            */
 
-/* Enqueue the chosen stages on the context stream; returns without waiting. */
+/* Enqueue the chosen stages on the context stream; returns without waiting.  The
+ * single stages may be captured into a graph of the caller's; from then on every run of
+ * that plan resets the work counters itself, since the graph may be replayed any time. */
 zmc_status zmc_plan_run(zmc_plan *plan, uint32_t stages);
 
 /* Enqueue the plain FP64 form (one launch per integrand + merge). */

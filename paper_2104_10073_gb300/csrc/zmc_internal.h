@@ -119,7 +119,9 @@ static_assert(sizeof(Entry) == 24, "Entry layout");
 // owns items [item_begin[f], item_end[f]) and is drained by its own persistent
 // kernel through counter[f].
 struct LaunchHdr {
-  unsigned long long counter[4];     // per-family item dispensers (zeroed before a launch)
+  // per-family item dispensers: zero when a launch starts (from the upload, the merge
+  // before it, or a reset)
+  unsigned long long counter[4];
   unsigned long long item_begin[4];
   unsigned long long item_end[4];
   uint32_t n_entries;

@@ -74,9 +74,9 @@ struct Eval<ZMC_USER, D, G> {
 #pragma unroll
     for (int i = 0; i < D; ++i) {
       // 1 + u from its bits by three integer operations, then an exact subtraction: one
-      // FP64 operation where the conversion and its scaling took two; the FP64 pipe
-      // (2 lanes an SM) is what bounds this kernel (100 rows of
-      // 10^5 samples, cos and sin of a 4-D phase: 1088 -> 1004 us)
+      // FP64 operation where the conversion and its scaling took two; the FP64 pipe is
+      // what bounds this kernel (100 rows of 10^5 samples, cos and sin of a 4-D phase:
+      // 1088 -> 1004 us)
       const double v = __hiloint2double(static_cast<int>(0x3FF00000u | ((r[i] >> 3) & 0xFFFFFu)),
                                         static_cast<int>(r[i] << 29));
       x[i] = fma(wd[i], v - 1.0, lo[i]);
