@@ -32,7 +32,10 @@ class Arena {
   void release(void *p);
   // Whether alloc(bytes) would succeed if these blocks were free.
   bool fits_without(const std::vector<void *> &blocks, size_t bytes) const;
-  size_t used() const { return used_; }
+  size_t used() const {
+    std::lock_guard<std::mutex> g(mu_);
+    return used_;
+  }
   size_t size() const { return size_; }
   size_t largest_free() const;
 
