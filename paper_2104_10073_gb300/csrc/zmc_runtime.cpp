@@ -1661,7 +1661,7 @@ zmc_status zmc_plan_device_results(zmc_plan *plan, void **device_ptr) {
 
 zmc_status zmc_plan_info_get(const zmc_plan *plan, zmc_plan_info *out) {
   if (!plan || !out) return set_error(ZMC_EINVAL, "null argument");
-  std::lock_guard<std::recursive_mutex> g(plan->ctx->api_mu);  // split_chunks may change
+  std::lock_guard<std::recursive_mutex> lock(plan->ctx->api_mu);  // split_chunks may change
   out->n_fn = plan->n;
   out->n_chunks = plan->n_chunks;
   out->n_samples = plan->n_samples;
